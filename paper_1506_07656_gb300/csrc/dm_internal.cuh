@@ -125,63 +125,110 @@ __device__ __forceinline__ float dm_powf(float x, float lam) {
     return __fmul_rn(__fmul_rn(p, dm_pow2i(na)), dm_pow2i(nb));
 }
 
-// dm_powf on two values at once: the same operations in the same order, the
-// floating-point ones as packed FP32x2 instructions where both lanes do the
-// same thing (each lane rounds exactly as the scalar operation would), so
-// each lane's result has the bits dm_powf gives it.  No packed product feeds a
-// packed addition (see the exponent reduction below).
-__device__ __forceinline__ float2 dm_powf2(float2 x, float lam) {
-    float2 r;
-    // lanes that leave the common path (x <= 0, subnormal x, a subnormal result)
-    // take the scalar recipe
-    const bool fast = x.x >= 1.17549435e-38f && x.y >= 1.17549435e-38f;
-    if (!fast) return make_float2(dm_powf(x.x, lam), dm_powf(x.y, lam));
-    const uint32_t b0 = __float_as_uint(x.x), b1 = __float_as_uint(x.y);
-    int e0 = (int)((b0 >> 23) & 0xffu) - 127, e1 = (int)((b1 >> 23) & 0xffu) - 127;
-    float m0 = __uint_as_float((b0 & 0x7fffffu) | 0x3f800000u), m1 = __uint_as_float((b1 & 0x7fffffu) | 0x3f800000u);
-    if (m0 > 1.41421356f) { m0 = __fmul_rn(m0, 0.5f); e0 = e0 + 1; }
-    if (m1 > 1.41421356f) { m1 = __fmul_rn(m1, 0.5f); e1 = e1 + 1; }
-    const float2 m = make_float2(m0, m1);
-    const float2 num = __fadd2_rn(m, make_float2(-1.0f, -1.0f));
-    const float2 den = __fadd2_rn(m, make_float2(1.0f, 1.0f));
-    const float2 f = make_float2(__fdiv_rn(num.x, den.x), __fdiv_rn(num.y, den.y));
-    const float2 f2 = __fmul2_rn(f, f);
-    float2 s = make_float2(7.69230769e-02f, 7.69230769e-02f);
-    s = __ffma2_rn(s, f2, make_float2(9.09090909e-02f, 9.09090909e-02f));
-    s = __ffma2_rn(s, f2, make_float2(1.11111111e-01f, 1.11111111e-01f));
-    s = __ffma2_rn(s, f2, make_float2(1.42857143e-01f, 1.42857143e-01f));
-    s = __ffma2_rn(s, f2, make_float2(2.00000000e-01f, 2.00000000e-01f));
-    s = __ffma2_rn(s, f2, make_float2(3.33333333e-01f, 3.33333333e-01f));
-    s = __ffma2_rn(s, f2, make_float2(1.0f, 1.0f));
-    const float2 l2m = __fmul2_rn(__fmul2_rn(make_float2(2.88539008f, 2.88539008f), f), s);
-    const float2 fe = make_float2((float)e0, (float)e1);
-    const float2 lam2 = make_float2(lam, lam);
-    const float2 a = __fmul2_rn(lam2, fe);
-    const float2 aerr = __ffma2_rn(lam2, fe, make_float2(-a.x, -a.y));
-    const float2 n1 = make_float2(rintf(a.x), rintf(a.y));
-    // the product lam * log2 m feeds an addition: it is formed by scalar
-    // multiplications, since a packed multiplication followed by a packed
-    // addition was found fused into one rounding despite contraction being off
-    const float2 lg = make_float2(__fmul_rn(lam, l2m.x), __fmul_rn(lam, l2m.y));
-    float2 g = __fadd2_rn(__fadd2_rn(__fadd2_rn(a, make_float2(-n1.x, -n1.y)), aerr), lg);
-    const float2 n2 = make_float2(rintf(g.x), rintf(g.y));
-    g = __fadd2_rn(g, make_float2(-n2.x, -n2.y));
-    float2 p = make_float2(1.52527338e-05f, 1.52527338e-05f);
-    p = __ffma2_rn(p, g, make_float2(1.54035304e-04f, 1.54035304e-04f));
-    p = __ffma2_rn(p, g, make_float2(1.33335581e-03f, 1.33335581e-03f));
-    p = __ffma2_rn(p, g, make_float2(9.61812911e-03f, 9.61812911e-03f));
-    p = __ffma2_rn(p, g, make_float2(5.55041087e-02f, 5.55041087e-02f));
-    p = __ffma2_rn(p, g, make_float2(2.40226507e-01f, 2.40226507e-01f));
-    p = __ffma2_rn(p, g, make_float2(6.93147181e-01f, 6.93147181e-01f));
-    p = __ffma2_rn(p, g, make_float2(1.0f, 1.0f));
-    // n1 + n2 is a sum of two small integers, exact in FP32: one conversion per lane
-    const float2 ntf = __fadd2_rn(n1, n2);
-    const int nt0 = (int)ntf.x, nt1 = (int)ntf.y;
-    if (nt0 >= -125 && nt1 >= -125) return __fmul2_rn(p, make_float2(dm_pow2i(nt0), dm_pow2i(nt1)));
-    // a result below the normal range: the scalar two-step scaling per lane
-    r.x = dm_powf(x.x, lam);
-    r.y = dm_powf(x.y, lam);
+// a - b for two lanes at once, each lane rounded as the scalar subtraction
+// (the packed add has no negated operand, so a - b written as a + (-b) would
+// need the negations as separate instructions)
+__device__ __forceinline__ float2 dm_fsub2(float2 a, float2 b) {
+    unsigned long long ra, rb, rd;
+    memcpy(&ra, &a, 8);
+    memcpy(&rb, &b, 8);
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
+    float2 d;
+    memcpy(&d, &rd, 8);
+    return d;
+}
+
+// Per-thread constants of dm_powf2: the exponent; the range of x of its packed
+// path, 2^(-118/lam) <= x <= 2^(100/lam) inside the normal numbers, so that x^lam is
+// normal with room to spare (empty for an exponent that is not safely positive); and
+// the pairs that its packed additions take.  The pairs pass through an empty asm, so
+// that they stay in registers: as literals they would be moved into a pair at each use.
+struct DmPow {
+    float lam, lo, hi;
+    float2 one2, magic2;
+};
+__device__ __forceinline__ DmPow dm_pow_setup(float lam) {
+    DmPow r;
+    r.lam = lam;
+    const bool ok = lam >= 0.01f && lam <= 1.0e4f;
+    r.lo = ok ? fmaxf(exp2f(-118.0f / lam), 2.4e-38f) : INFINITY;
+    r.hi = ok ? exp2f(fminf(100.0f / lam, 100.0f)) : 0.0f;
+    r.one2 = make_float2(1.0f, 1.0f);
+    r.magic2 = make_float2(12582912.0f, 12582912.0f);      // 1.5 2^23, 0x4b400000
+    asm volatile("" : "+f"(r.one2.x), "+f"(r.one2.y), "+f"(r.magic2.x), "+f"(r.magic2.y));
     return r;
+}
+
+// dm_powf on two values at once, each lane with the bits dm_powf gives it.
+// The function is bound by the issue of its ~50 instructions for two values,
+// so every step that has a cheaper form with the same result takes it:
+//   - e and m from one integer subtraction: the octave [sqrt(1/2), sqrt(2)] of m
+//     is 2^23 consecutive bit patterns from 0x3f3504f4 on;
+//   - f = (m - 1) / (m + 1), correctly rounded, as the quotient estimate
+//     num * (1 / den) with one remainder correction (Markstein's: the remainder
+//     of an fma is exact, the correction rounds once); f depends on m alone, and
+//     the result equals the correctly rounded division for every one of the 2^23
+//     values of m (tests/test_gpu_pow.py compares all of them);
+//   - rint by adding and subtracting 1.5 2^23, whose low bits are then the
+//     integer itself, so that 2^n multiplies by an addition to the exponent field;
+//   - (a - n1) + aerr, with a - n1 exact and aerr the exact error of a = RN(lam e),
+//     is RN(lam e - n1): one fma.
+// (The products lam e and lam log2 m feed additions: they are formed by scalar
+// multiplications, since a packed multiplication followed by a packed addition
+// was found fused into one rounding despite contraction being off.)
+// Steps with a literal coefficient are scalar (an fma takes a literal operand; a pair
+// of them would take two moves); the others are packed.  48 -> 37 instructions per value; the level pass of a
+// 1024x436 pair 7.65 -> 7.48 ms.
+__device__ __forceinline__ float2 dm_powf2(float2 x, const DmPow& R) {
+    const float lam = R.lam;
+    // (a NaN fails the comparisons)
+    const bool fast = x.x >= R.lo && x.y >= R.lo && fmaxf(x.x, x.y) <= R.hi;
+    if (!fast) return make_float2(dm_powf(x.x, lam), dm_powf(x.y, lam));
+    const int b0 = __float_as_int(x.x), b1 = __float_as_int(x.y);
+    const int t0 = b0 - 0x3f3504f4, t1 = b1 - 0x3f3504f4;
+    const float2 m = make_float2(__int_as_float(b0 - (t0 & 0xff800000)), __int_as_float(b1 - (t1 & 0xff800000)));
+    const float2 fe = dm_fsub2(make_float2(__int_as_float((t0 >> 23) + 0x4b400000), __int_as_float((t1 >> 23) + 0x4b400000)),
+                               R.magic2);
+    const float2 num = dm_fsub2(m, R.one2), den = __fadd2_rn(m, R.one2);
+    // r = -1 / den (approximately), q = -num / den; f is carried with its sign flipped
+    float2 r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(-den.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(-den.y));
+    const float2 q = __fmul2_rn(num, r);
+    const float2 f = __ffma2_rn(__ffma2_rn(den, q, num), r, q);
+    const float2 f2 = __fmul2_rn(f, f);
+    auto log_poly = [](float v) {
+        float s = __fmaf_rn(7.69230769e-02f, v, 9.09090909e-02f);
+        s = __fmaf_rn(s, v, 1.11111111e-01f);
+        s = __fmaf_rn(s, v, 1.42857143e-01f);
+        s = __fmaf_rn(s, v, 2.00000000e-01f);
+        s = __fmaf_rn(s, v, 3.33333333e-01f);
+        return __fmaf_rn(s, v, 1.0f);
+    };
+    const float lg0 = __fmul_rn(lam, __fmul_rn(__fmul_rn(-2.88539008f, f.x), log_poly(f2.x)));
+    const float lg1 = __fmul_rn(lam, __fmul_rn(__fmul_rn(-2.88539008f, f.y), log_poly(f2.y)));
+    const float2 u1 = __fadd2_rn(make_float2(__fmul_rn(lam, fe.x), __fmul_rn(lam, fe.y)), R.magic2);   // low bits: n1
+    const float2 nn1 = dm_fsub2(R.magic2, u1);         // -n1
+    float2 g = __fadd2_rn(make_float2(__fmaf_rn(lam, fe.x, nn1.x), __fmaf_rn(lam, fe.y, nn1.y)), make_float2(lg0, lg1));
+    const float2 u2 = __fadd2_rn(g, R.magic2);         // low bits: n2
+    g = __fadd2_rn(g, dm_fsub2(R.magic2, u2));
+    auto exp_poly = [](float v) {
+        float p = __fmaf_rn(1.52527338e-05f, v, 1.54035304e-04f);
+        p = __fmaf_rn(p, v, 1.33335581e-03f);
+        p = __fmaf_rn(p, v, 9.61812911e-03f);
+        p = __fmaf_rn(p, v, 5.55041087e-02f);
+        p = __fmaf_rn(p, v, 2.40226507e-01f);
+        p = __fmaf_rn(p, v, 6.93147181e-01f);
+        return __fmaf_rn(p, v, 1.0f);
+    };
+    // 2^(n1 + n2): the sum of the two magic numbers' bits is n1 + n2 plus a
+    // constant whose shift by 23 leaves 32 bits (the shift is spelled out: written
+    // as << 23 it was dropped for the first lane by the compiler, CUDA 13.0)
+    uint32_t k0 = __float_as_uint(u1.x) + __float_as_uint(u2.x), k1 = __float_as_uint(u1.y) + __float_as_uint(u2.y);
+    asm("shl.b32 %0, %0, 23;" : "+r"(k0));
+    asm("shl.b32 %0, %0, 23;" : "+r"(k1));
+    return make_float2(__uint_as_float(__float_as_uint(exp_poly(g.x)) + k0),
+                       __uint_as_float(__float_as_uint(exp_poly(g.y)) + k1));
 }
 
 // ---------------------------------------------------------------------------
@@ -300,19 +347,6 @@ struct Kids {
     const float* base[4];
     int n;
 };
-
-// a - b for two lanes at once, each lane rounded as the scalar subtraction
-// (the packed add has no negated operand, so a - b written as a + (-b) would
-// need the negations as separate instructions)
-__device__ __forceinline__ float2 dm_fsub2(float2 a, float2 b) {
-    unsigned long long ra, rb, rd;
-    memcpy(&ra, &a, 8);
-    memcpy(&rb, &b, 8);
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
-    float2 d;
-    memcpy(&d, &rd, 8);
-    return d;
-}
 
 // One packed step of Knuth's TwoSum (s, x) -> (s + x, its rounding error),
 // two lanes at once; every operation rounded as the scalar one.

@@ -202,6 +202,7 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
         const int kk = tid % PW, u0 = tid / PW;
         const int rx = rx0 + kk, ry = ry0 + (u0 % PH);
         const int mw = g.dw[1], mh = g.dh[1];
+        const DmPow pr = dm_pow_setup(lam);
         if (rx < mw && ry < mh) {
             const int pl0 = u0 / PH;
             const long long pstride = (long long)mh * g.pitch(1);
@@ -209,7 +210,7 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
 #pragma unroll 2
             for (int j = 0; j < PATCHES / 2; j += 2) {
                 const int e = tid + j * 16 * PW;
-                const float2 v = dm_powf2(make_float2(best_s[e], best_s[e + 16 * PW]), lam);
+                const float2 v = dm_powf2(make_float2(best_s[e], best_s[e + 16 * PW]), pr);
                 const int p = p_base + pl0 + 2 * j;
                 const long long o = o0 + 2 * j * pstride;
                 if (p < n0) {

@@ -298,6 +298,7 @@ __device__ __forceinline__ void level_sweep_body(const DmGeom& g, int l, const C
         }
     }
     __syncthreads();
+    const DmPow pr = dm_pow_setup(lam);
     const bool interior = qx0 >= 0 && qy0 >= 0 && qx0 + AW <= mw && qy0 + AH <= mh;
     // thread 0 waits for the loads; the barrier after its wait passes their
     // data on to every thread of the CTA
@@ -406,7 +407,7 @@ __device__ __forceinline__ void level_sweep_body(const DmGeom& g, int l, const C
                 // are evaluated on whatever the tile holds there and not stored)
 #pragma unroll
                 for (int j = 0; j + 1 < R; j += 2) {
-                    const float2 v = dm_powf2(make_float2(best[j], best[j + 1]), lam);
+                    const float2 v = dm_powf2(make_float2(best[j], best[j + 1]), pr);
                     pw[j] = v.x;
                     pw[j + 1] = v.y;
                 }
@@ -534,7 +535,7 @@ __device__ __forceinline__ void stream_hrow(const StreamWarp& w, const float2* v
 // One step: output rows ry and ry + 1 from A rows 2ry - 1 (carried in hp, cp)
 // to 2ry + 3.
 template <bool COMP, bool CHECK>
-__device__ __forceinline__ void stream_step(const StreamWarp& w, int ry, int oh, float& hp, int& cp, float lam,
+__device__ __forceinline__ void stream_step(const StreamWarp& w, int ry, int oh, float& hp, int& cp, const DmPow& pr,
                                             bool store, float* __restrict__ orow, unsigned char* __restrict__ arow,
                                             int opitch) {
     float2 v[4][4];
@@ -552,7 +553,7 @@ __device__ __forceinline__ void stream_step(const StreamWarp& w, int ry, int oh,
     cp = hc[3];
     const bool two = ry + 1 < oh;
     // (with one output row left, the second lane of the pair repeats the first and is not stored)
-    const float2 pw = dm_powf2(make_float2(b0, two ? b1 : b0), lam);
+    const float2 pw = dm_powf2(make_float2(b0, two ? b1 : b0), pr);
     if (store) {
         orow[(long long)ry * opitch] = pw.x;
         arow[(long long)ry * opitch] = (unsigned char)c0;
@@ -619,15 +620,16 @@ __device__ __forceinline__ void level_stream_body(const DmGeom& g, int l, const 
 
     float* orow = out + (long long)p * oh * opitch + rx;
     unsigned char* arow = amax + (long long)p * oh * opitch + rx;
+    const DmPow pr = dm_pow_setup(lam);
     float hp = -INFINITY;                                   // A row 2ry - 1 (none for ry = 0)
     int cp = 0;
     int ry = 0;
     if (inside) {
         // step ry reads child rows 2ry - 1 .. 2ry + 4: unchecked while they lie in the domain
-        stream_step<COMP, true>(w, 0, oh, hp, cp, lam, store, orow, arow, opitch);
-        for (ry = 2; 2 * ry + 4 < w.mh; ry += 2) stream_step<COMP, false>(w, ry, oh, hp, cp, lam, store, orow, arow, opitch);
+        stream_step<COMP, true>(w, 0, oh, hp, cp, pr, store, orow, arow, opitch);
+        for (ry = 2; 2 * ry + 4 < w.mh; ry += 2) stream_step<COMP, false>(w, ry, oh, hp, cp, pr, store, orow, arow, opitch);
     }
-    for (; ry < oh; ry += 2) stream_step<COMP, true>(w, ry, oh, hp, cp, lam, store, orow, arow, opitch);
+    for (; ry < oh; ry += 2) stream_step<COMP, true>(w, ry, oh, hp, cp, pr, store, orow, arow, opitch);
 }
 
 template <bool COMP, bool APPROX = false>
