@@ -33,6 +33,8 @@
 // map zero-fills whatever lies outside the domain.)  Algorithmic bytes per
 // stored output: 16 B of child values read (each child value is shared by 4
 // parents), 4 + 1 B written.
+#include <algorithm>
+
 #include "dm_internal.cuh"
 
 namespace {
@@ -441,206 +443,312 @@ __global__ void __launch_bounds__(NT) k_level_sweep(DmGeom g, int l, const __gri
 }
 
 // ---------------------------------------------------------------------------
-// Row-streaming form of the same pass (level_th = 0 in the tuned shapes).
+// Row-streaming form of the same pass: a warp walks down the rows of its patches'
+// maps in registers, with no shared memory and no barrier but a rare one.
 //
-// One warp owns one lattice patch p and a strip of STREAM_W = 31 pooled columns
-// [r0, r0 + 31) of its stored map, and walks down every row of it: no shared
-// memory, no barrier.  For a row y of averages, lane t forms A(2(r0+t) - 1, y)
-// and A(2(r0+t), y), two columns at once with the packed child sum: the
-// children with o_x = -1 contribute their columns 2(r0+t) - 2 and - 1, those
-// with o_x = +1 their columns 2(r0+t) and + 1 -- one aligned 8-byte load per
-// child, from row y - 1 (o_y = -1) or y + 1 (o_y = +1).  A(2(r0+t) + 1, y) is
-// lane t+1's first average (one shuffle); lane 31 only supplies it.  The
-// horizontal 3-maxima of the rows stay in registers and merge over three rows
-// into the pooled output, two output rows per step (one packed power).
-// Missing children and samples outside the domain read as 0, which leaves both
-// child sums unchanged (s + 0 = s exactly, with a zero TwoSum error), so every
-// patch runs the four-child arithmetic and divides by its number of children;
-// warps whose strip and children lie wholly inside take loads without any
-// masks, and only the first and last steps check rows.  The 8 warps of a CTA
-// take a 4 x 2 block of patches spaced S apart, which share child maps: each
-// child row a CTA needs comes from L2 once and is reused from L1.
-// ---------------------------------------------------------------------------
-constexpr int STREAM_W = 31;        // pooled columns per warp strip
-constexpr int STREAM_BX = 4, STREAM_BY = 2;   // patches per CTA along x and y
-constexpr int STREAM_WARPS = STREAM_BX * STREAM_BY;
+// What bounds it: at level 1 of a 1024x436 pair 167 instructions per output at 66 %
+// issue, the rest the latency of the child loads (62 % L1 hits; DRAM reads 1.19x the
+// maps, 59 % of the copy bandwidth with the writes); 4.49 ms against 5.36 ms of the
+// tiled kernel, whose averages go through shared memory between two barriers per patch.
+// Also measured there (whole level pass, this form 6.24 ms): the next rows' loads held in
+// registers (2 CTAs per SM) 7.8, the child rows staged by 4-D TMA loads of two rows of
+// every map 8.2 (a load costs about 45 cycles per map it touches), staged by 16-byte
+// asynchronous copies 8.9, all strips of a row in one CTA 6.7.
+//
+// Work split of level l.  A unit of LPP lanes (32, 16, 8 or 4) owns one lattice
+// patch and a strip of 2 LPP pooled columns; a warp holds 32 / LPP units of
+// neighbouring patches, so that narrow maps fill their lanes too.  A lane owns two
+// neighbouring pooled columns and the four columns of averages they need (the fifth
+// is the next lane's first).  A CTA of 4 x 2 warps owns a block of patches spaced
+// S = 2^(l-1) apart (1 at level 1), which share their child maps: the right children
+// of one patch are the left children of the next, likewise up and down, so 4 x 2
+// patches read 15 maps instead of 32 and the rest hits in L1.  It walks down a
+// segment of rows.  CTAs are numbered in groups of LV_GROUP along x, then the strips
+// (which share the memory sectors at their edges), then the rows of patches, then the
+// groups and the segments: the child rows that two rows of patches share are still in
+// L2 when the second one reads them (level pass 6.60 ms with all of a row of patches
+// first, 6.66 with the strips after the rows of patches, 6.34 so).
+constexpr int LV_GROUP = 16;        // CTAs along x numbered together (see level_shape)
+constexpr int LV_WX = 4, LV_WY = 2;  // warps of a CTA
+constexpr int LV_THREADS = 32 * LV_WX * LV_WY;
 
-// Average of the four children (child order i = 0..3, zeros for missing ones)
-// for two columns at once, then times 1/n (n = 3 divides).
+__host__ __device__ constexpr int level_stride(int l) { return l == 1 ? 1 : 1 << (l - 1); }
+
+// One row of averages of a lane: columns q0 - 1 .. q0 + 2, then the next
+// lane's first (q0 + 3), and the horizontal 3-maxima of the two pooled columns.
+struct LvRow {
+    float a[5];
+    float h0, h1;
+};
+
+// The child values of one row of averages: per child side the left pair of
+// children's columns q0 - 2 .. q0 + 1 (o_x = -1) and the right pair's q0 .. q0 + 3.
+struct LvKids {
+    float2 lt0, lt1, lb0, lb1;
+    float4 rt, rb;
+};
+
+// Average of the four children (child order: left top, left bottom, right top,
+// right bottom; zeros for missing ones leave the sums unchanged: s + 0 = s, with
+// a zero error) for two columns at once, times w = 1 / n.  The compensated sum's
+// first FAST steps take Dekker's Fast2Sum on (max, min), the others Knuth's
+// TwoSum: both give the exact rounding error of a sum of non-negative values,
+// hence the same bits.  TwoSum costs 3 instructions per value and step on the
+// FP32 pipe alone; Fast2Sum 3.5, 2 of them min / max on the integer pipe, which
+// is idle here.
+template <bool FAST>
+__device__ __forceinline__ void lv_two_sum(float2& s, float2 x, float2& err) {
+    if constexpr (FAST) {
+        const float2 hi = make_float2(fmaxf(s.x, x.x), fmaxf(s.y, x.y)), lo = make_float2(fminf(s.x, x.x), fminf(s.y, x.y));
+        const float2 t = __fadd2_rn(s, x);
+        err = dm_fsub2(lo, dm_fsub2(t, hi));
+        s = t;
+    } else {
+        dm_two_sum2(s, x, err);
+    }
+}
+
+constexpr int LV_FAST_STEPS = 2;
 template <bool COMP>
-__device__ __forceinline__ float2 avg_pair(const float2* v, int n) {
-    float2 sv = v[0];
+__device__ __forceinline__ float2 lv_avg2(float2 x0, float2 x1, float2 x2, float2 x3, float w) {
+    float2 sv = x0;
     if constexpr (COMP) {
-        float2 cp = make_float2(0.0f, 0.0f);
-#pragma unroll
-        for (int i = 1; i < 4; i++) {
-            float2 err;
-            dm_two_sum2(sv, v[i], err);
-            cp = i == 1 ? err : __fadd2_rn(cp, err);
-        }
+        float2 cp, err;
+        lv_two_sum<(LV_FAST_STEPS > 0)>(sv, x1, cp);
+        lv_two_sum<(LV_FAST_STEPS > 1)>(sv, x2, err);
+        cp = __fadd2_rn(cp, err);
+        lv_two_sum<(LV_FAST_STEPS > 2)>(sv, x3, err);
+        cp = __fadd2_rn(cp, err);
         sv = __fadd2_rn(sv, cp);
     } else {
-#pragma unroll
-        for (int i = 1; i < 4; i++) sv = __fadd2_rn(sv, v[i]);
+        sv = __fadd2_rn(__fadd2_rn(__fadd2_rn(sv, x1), x2), x3);
     }
-    if (n == 4) return __fmul2_rn(sv, make_float2(0.25f, 0.25f));
-    if (n == 3) return make_float2(__fdiv_rn(sv.x, 3.0f), __fdiv_rn(sv.y, 3.0f));
-    const float w = n == 2 ? 0.5f : 1.0f;
     return __fmul2_rn(sv, make_float2(w, w));
 }
 
-// Per-warp state of the row-streaming kernel.
-struct StreamWarp {
-    const float* kid[4];   // child maps (nullptr: missing)
-    int n;                 // existing children
-    int mw, mh, pitch;     // child map domain and row pitch (level l)
-    int xl, xr;            // first column of this lane's left / right child pairs
-    int ml, mr;            // their load modes: 3 both columns in the domain, 1 only the first, 0 none
-    bool has_a0, has_a2;   // A(2rx - 1) and A(2rx + 1) in the domain
+// Per-lane state of the kernel.
+struct LvLane {
+    const char* kid[4];     // child maps (nullptr: missing)
+    float w;                // 1 / number of children
+    int mw, mh;             // child map domain (level l)
+    uint32_t pitch4;        // row pitch in bytes
+    int q0;                 // 2 x the lane's first pooled column
+    bool first;             // q0 == 0: column -1 does not exist
 };
 
-// The four children's pairs of A row y.  CHECK: rows outside the domain, missing
-// children and columns outside the domain read as zeros; otherwise every load is
-// known to be inside.
-template <bool CHECK>
-__device__ __forceinline__ void stream_load_row(const StreamWarp& w, float2* v, int y) {
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        const int cy = y + ((i & 1) ? 1 : -1);
-        const int x = i < 2 ? w.xl : w.xr;
-        if constexpr (!CHECK) {
-            v[i] = __ldg(reinterpret_cast<const float2*>(w.kid[i] + (cy * w.pitch + x)));
-        } else {
-            const int mode = i < 2 ? w.ml : w.mr;
-            const bool ok = w.kid[i] != nullptr && cy >= 0 && cy < w.mh;
-            float2 t = make_float2(0.0f, 0.0f);
-            if (ok && mode == 3) t = __ldg(reinterpret_cast<const float2*>(w.kid[i] + (cy * w.pitch + x)));
-            else if (ok && mode == 1) t.x = __ldg(w.kid[i] + (cy * w.pitch + x));
-            v[i] = t;
-        }
+// Child values of average row y; `off32` is the byte offset of (row y - 1,
+// column q0) in a child map.  IN: every child exists, the rows y - 1, y + 1 and the lane's
+// columns lie inside the maps (column -2 of the first lane is the padding before
+// the row, whose values are replaced; y - 1 >= 1 there).  Otherwise missing
+// children and rows and columns outside the domain read as zeros; a vector whose
+// first element lies inside the domain lies inside the row's padded pitch, so it is
+// loaded whole and its elements past the domain are replaced.
+template <bool IN>
+__device__ __forceinline__ LvKids lv_load(const LvLane& L, int y, uint32_t off32) {
+    LvKids v;
+    if constexpr (IN) {
+        const uint32_t ot = off32, ob = ot + 2u * L.pitch4;
+        v.lt0 = __ldg(reinterpret_cast<const float2*>(L.kid[0] + ot - 8));
+        v.lt1 = __ldg(reinterpret_cast<const float2*>(L.kid[0] + ot));
+        v.lb0 = __ldg(reinterpret_cast<const float2*>(L.kid[1] + ob - 8));
+        v.lb1 = __ldg(reinterpret_cast<const float2*>(L.kid[1] + ob));
+        v.rt = __ldg(reinterpret_cast<const float4*>(L.kid[2] + ot));
+        v.rb = __ldg(reinterpret_cast<const float4*>(L.kid[3] + ob));
+    } else {
+        const size_t off = (size_t)((long long)(y - 1) * L.pitch4 + 4LL * L.q0), ob = off + 2u * (size_t)L.pitch4;
+        const bool t = y >= 1 && y <= L.mh, b = y >= -1 && y + 1 < L.mh;
+        const bool c0 = L.q0 < L.mw, cl = !L.first && L.q0 - 2 < L.mw;
+        const float2 z2 = make_float2(0.0f, 0.0f);
+        const float4 z4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        v.lt0 = t && cl && L.kid[0] ? __ldg(reinterpret_cast<const float2*>(L.kid[0] + off - 8)) : z2;
+        v.lt1 = t && c0 && L.kid[0] ? __ldg(reinterpret_cast<const float2*>(L.kid[0] + off)) : z2;
+        v.lb0 = b && cl && L.kid[1] ? __ldg(reinterpret_cast<const float2*>(L.kid[1] + ob - 8)) : z2;
+        v.lb1 = b && c0 && L.kid[1] ? __ldg(reinterpret_cast<const float2*>(L.kid[1] + ob)) : z2;
+        v.rt = t && c0 && L.kid[2] ? __ldg(reinterpret_cast<const float4*>(L.kid[2] + off)) : z4;
+        v.rb = b && c0 && L.kid[3] ? __ldg(reinterpret_cast<const float4*>(L.kid[3] + ob)) : z4;
+        if (L.q0 - 1 >= L.mw) { v.lt0.y = 0.0f; v.lb0.y = 0.0f; }
+        if (L.q0 + 1 >= L.mw) { v.lt1.y = 0.0f; v.lb1.y = 0.0f; v.rt.y = 0.0f; v.rb.y = 0.0f; }
+        if (L.q0 + 2 >= L.mw) { v.rt.z = 0.0f; v.rb.z = 0.0f; }
+        if (L.q0 + 3 >= L.mw) { v.rt.w = 0.0f; v.rb.w = 0.0f; }
     }
+    return v;
 }
 
-// Horizontal 3-max (first column equal to the maximum) of A row y; -inf outside the domain.
+// The average at (x, y) (scalar, the same sums), -inf outside the domain: the
+// column right of a unit's last lane (x >= 1), one row per lane.
 template <bool COMP>
-__device__ __forceinline__ void stream_hrow(const StreamWarp& w, const float2* v, int y, float& h, int& hc) {
-    const float2 a = avg_pair<COMP>(v, w.n);
-    const float a2s = __shfl_down_sync(0xffffffffu, a.x, 1);
-    const float a0 = w.has_a0 ? a.x : -INFINITY, a1 = a.y, a2 = w.has_a2 ? a2s : -INFINITY;
-    const float m = fmax3(a0, a1, a2);
-    h = y < w.mh ? m : -INFINITY;
-    hc = a0 == m ? 0 : (a1 == m ? 1 : 2);
+__device__ __forceinline__ float lv_extra(const LvLane& L, int y, int x) {
+    const bool t = y >= 1, b = y + 1 < L.mh, r = x + 1 < L.mw;
+    if (y < 0 || y >= L.mh || x >= L.mw) return -INFINITY;
+    const size_t ot = (size_t)(y - 1) * L.pitch4 + (size_t)x * 4, ob = ot + 2u * (size_t)L.pitch4;
+    const float v0 = t && L.kid[0] ? __ldg(reinterpret_cast<const float*>(L.kid[0] + ot - 4)) : 0.0f;
+    const float v1 = b && L.kid[1] ? __ldg(reinterpret_cast<const float*>(L.kid[1] + ob - 4)) : 0.0f;
+    const float v2 = t && r && L.kid[2] ? __ldg(reinterpret_cast<const float*>(L.kid[2] + ot + 4)) : 0.0f;
+    const float v3 = b && r && L.kid[3] ? __ldg(reinterpret_cast<const float*>(L.kid[3] + ob + 4)) : 0.0f;
+    float s = v0, comp = 0.0f;
+    child_add<COMP>(s, comp, v1);
+    child_add<COMP>(s, comp, v2);
+    child_add<COMP>(s, comp, v3);
+    return __fmul_rn(__fadd_rn(s, comp), L.w);
 }
 
-// One step: output rows ry and ry + 1 from A rows 2ry - 1 (carried in hp, cp)
-// to 2ry + 3.
-template <bool COMP, bool CHECK>
-__device__ __forceinline__ void stream_step(const StreamWarp& w, int ry, int oh, float& hp, int& cp, const DmPow& pr,
-                                            bool store, float* __restrict__ orow, unsigned char* __restrict__ arow,
-                                            int opitch) {
-    float2 v[4][4];
+// Averages and horizontal maxima of one row from its child values; `ex` holds the
+// unit's extra column for the row in lane `src` of the unit.
+template <bool COMP, bool IN, int LPP>
+__device__ __forceinline__ LvRow lv_row(const LvLane& L, LvKids v, int y, float ex, int src) {
+    LvRow r;
+    if constexpr (IN)
+        if (L.first) { v.lt0.y = 0.0f; v.lb0.y = 0.0f; }
+    const float2 a01 = lv_avg2<COMP>(v.lt0, v.lb0, make_float2(v.rt.x, v.rt.y), make_float2(v.rb.x, v.rb.y), L.w);
+    const float2 a23 = lv_avg2<COMP>(v.lt1, v.lb1, make_float2(v.rt.z, v.rt.w), make_float2(v.rb.z, v.rb.w), L.w);
+    r.a[0] = L.first ? -INFINITY : a01.x;
+    r.a[1] = a01.y;
+    r.a[2] = a23.x;
+    r.a[3] = a23.y;
+    if constexpr (!IN) {
+        const bool in = y >= 0 && y < L.mh;
 #pragma unroll
-    for (int k = 0; k < 4; k++) stream_load_row<CHECK>(w, v[k], 2 * ry + k);
-    float h[4];
-    int hc[4];
-#pragma unroll
-    for (int k = 0; k < 4; k++) stream_hrow<COMP>(w, v[k], 2 * ry + k, h[k], hc[k]);
-    const float b0 = fmax3(hp, h[0], h[1]);
-    const int c0 = hp == b0 ? cp : (h[0] == b0 ? 3 + hc[0] : 6 + hc[1]);
-    const float b1 = fmax3(h[1], h[2], h[3]);
-    const int c1 = h[1] == b1 ? hc[1] : (h[2] == b1 ? 3 + hc[2] : 6 + hc[3]);
-    hp = h[3];
-    cp = hc[3];
-    const bool two = ry + 1 < oh;
-    // (with one output row left, the second lane of the pair repeats the first and is not stored)
-    const float2 pw = dm_powf2(make_float2(b0, two ? b1 : b0), pr);
-    if (store) {
-        orow[(long long)ry * opitch] = pw.x;
-        arow[(long long)ry * opitch] = (unsigned char)c0;
-        if (two) {
-            orow[(long long)(ry + 1) * opitch] = pw.y;
-            arow[(long long)(ry + 1) * opitch] = (unsigned char)c1;
-        }
+        for (int j = 0; j < 4; j++)
+            if (!in || L.q0 - 1 + j >= L.mw) r.a[j] = -INFINITY;
     }
+    const float nx = __shfl_down_sync(0xffffffffu, r.a[0], 1, LPP);
+    const float e = __shfl_sync(0xffffffffu, ex, src, LPP);
+    r.a[4] = (threadIdx.x & (LPP - 1)) == LPP - 1 ? e : nx;
+    r.h0 = fmax3(r.a[0], r.a[1], r.a[2]);
+    r.h1 = fmax3(r.a[2], r.a[3], r.a[4]);
+    return r;
 }
 
-template <bool COMP, bool APPROX>
-__device__ __forceinline__ void level_stream_body(const DmGeom& g, int l, const float* __restrict__ prev,
-                                                  const unsigned char* __restrict__ vprev,
-                                                  const unsigned char* __restrict__ vcur, int bx_per_res, int by_per_res,
-                                                  float* __restrict__ out, unsigned char* __restrict__ amax, float lam,
-                                                  const int* __restrict__ proto_of, int n_maps, long long item) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int cx0, cy0, S;
-    child_col_row(g, l, 0, 0, &cx0, &cy0, &S);
-    // block = (((strip * S + res_y) * by_per_res + by) * S + res_x) * bx_per_res + bx: a block holds
-    // patches (res_x + (bx * 4 + wx) S, res_y + (by * 2 + wy) S), wx < 4, wy < 2
-    const int bx = (int)(item % bx_per_res);
-    item /= bx_per_res;
-    const int res_x = (int)(item % S);
-    item /= S;
-    const int by = (int)(item % by_per_res);
-    item /= by_per_res;
-    const int res_y = (int)(item % S);
-    const int strip = (int)(item / S);
-    const int ix = res_x + (bx * STREAM_BX + (warp % STREAM_BX)) * S;
-    const int iy = res_y + (by * STREAM_BY + (warp / STREAM_BX)) * S;
-    if (ix >= g.Lx || iy >= g.Ly) return;
-    const int p = iy * g.Lx + ix;
-    if (!vcur[p]) return;
+// Maximum of the 3x3 window whose columns start at a[C] of the rows r0, r1, r2, and
+// its code: the first row holding the maximum (m_y = -1, 0, 1), then the first
+// column of that row holding it: the first maximum in scan order.
+template <int C>
+__device__ __forceinline__ float lv_pool(const LvRow& r0, const LvRow& r1, const LvRow& r2, uint32_t& code) {
+    const float h0 = C ? r0.h1 : r0.h0, h1 = C ? r1.h1 : r1.h0, h2 = C ? r2.h1 : r2.h0;
+    const float b = fmax3(h0, h1, h2);
+    const bool p0 = h0 == b, p1 = h1 == b;
+    const float x0 = p0 ? r0.a[C] : (p1 ? r1.a[C] : r2.a[C]);
+    const float x1 = p0 ? r0.a[C + 1] : (p1 ? r1.a[C + 1] : r2.a[C + 1]);
+    code = (p0 ? 0u : (p1 ? 3u : 6u)) + (x0 == b ? 0u : (x1 == b ? 1u : 2u));
+    return b;
+}
 
-    StreamWarp w;
-    w.mw = g.dw[l];
-    w.mh = g.dh[l];
-    w.pitch = g.pitch(l);
+template <bool COMP, int LPP>
+__device__ __forceinline__ void level_rows_body(const DmGeom& g, int l, const float* __restrict__ prev,
+                                                const unsigned char* __restrict__ vprev, int nbx, int nby, int seg_rows,
+                                                float* __restrict__ out, unsigned char* __restrict__ amax, float lam,
+                                                const int* __restrict__ proto_of, int n_maps, unsigned item) {
+    constexpr int UPW = 32 / LPP;                            // units per warp
+    const int lane = threadIdx.x & 31, ul = lane & (LPP - 1);
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // warp-uniform
     const int ow = g.dw[l + 1], oh = g.dh[l + 1], opitch = g.pitch(l + 1);
-    const long long csize = g.psize(l);
-    w.n = 0;
+
+    const int S = level_stride(l), strips = (ow + 2 * LPP - 1) / (2 * LPP);
+    // numbering of the CTAs: see level_shape
+    const unsigned nbxs = (unsigned)(S * nbx), nbys = (unsigned)(S * nby), per = nbys * (unsigned)(strips * LV_GROUP);
+    const unsigned groups = (nbxs + LV_GROUP - 1) / LV_GROUP;
+    unsigned t = item;
+    const int seg = (int)(t / (per * groups));
+    t -= (unsigned)seg * per * groups;
+    const unsigned grp = t / per;
+    t -= grp * per;
+    const int byi = (int)(t / (unsigned)(strips * LV_GROUP));
+    t -= (unsigned)byi * (unsigned)(strips * LV_GROUP);
+    const int strip = (int)(t / LV_GROUP), bxi = (int)(grp * LV_GROUP + t % LV_GROUP);
+    if (bxi >= (int)nbxs) return;                            // (the whole CTA)
+    // residues slowest: consecutive blocks of a residue share child maps
+    const int res_x = bxi / nbx, res_y = byi / nby;
+    const int ix = res_x + (((bxi - res_x * nbx) * LV_WX + (warp & (LV_WX - 1))) * UPW + (LPP == 32 ? 0 : lane / LPP)) * S;
+    const int iy = res_y + ((byi - res_y * nby) * LV_WY + warp / LV_WX) * S;
+    const int p = iy * g.Lx + ix;
+
+    LvLane L;
+    L.mw = g.dw[l];
+    L.mh = g.dh[l];
+    L.pitch4 = (uint32_t)g.pitch(l) * 4u;
+    L.q0 = 4 * (strip * LPP + ul);
+    L.first = L.q0 == 0;
+    const size_t csize = (size_t)g.psize(l);
+    int n = 0;
 #pragma unroll
     for (int i = 0; i < 4; i++) {
-        const int c = dm_child(g, l, ix, iy, i);
-        w.kid[i] = nullptr;
+        const int c = (ix < g.Lx && iy < g.Ly) ? dm_child(g, l, ix, iy, i) : -1;
+        L.kid[i] = nullptr;
         if (c >= 0 && vprev[c]) {
-            const int cm = APPROX ? min(max(__ldg(proto_of + c), 0), n_maps - 1) : c;
-            w.kid[i] = prev + (long long)cm * csize;
-            w.n++;
+            const int cm = proto_of ? min(max(__ldg(proto_of + c), 0), n_maps - 1) : c;
+            L.kid[i] = reinterpret_cast<const char*>(prev + (size_t)cm * csize);
+            n++;
         }
     }
-    const int r0 = strip * STREAM_W, rx = r0 + lane;
-    w.xl = 2 * rx - 2;
-    w.xr = 2 * rx;
-    auto mode_of = [&](int x) { return (x >= 0 && x < w.mw) ? ((x + 1 < w.mw) ? 3 : 1) : 0; };
-    w.ml = mode_of(w.xl);
-    w.mr = mode_of(w.xr);
-    w.has_a0 = rx >= 1;
-    w.has_a2 = 2 * rx + 1 < w.mw;
-    const bool store = lane < STREAM_W && rx < ow;
-    // every lane's pairs inside the domain and all four children present
-    const bool inside = w.n == 4 && 2 * r0 - 2 >= 0 && 2 * (r0 + 31) + 1 < w.mw;
-
-    float* orow = out + (long long)p * oh * opitch + rx;
-    unsigned char* arow = amax + (long long)p * oh * opitch + rx;
+    // existence factorises into columns times rows (the four children are two
+    // columns times two rows, level by level), so n is 0, 1, 2 or 4
+    L.w = n == 4 ? 0.25f : (n == 2 ? 0.5f : 1.0f);
+    const bool any = __any_sync(0xffffffffu, n > 0);
+    // every unit of the warp has all its children and a complete strip (and byte
+    // offsets within a map fit 32 bits): rows inside the map need no checks
+    const bool full = __all_sync(0xffffffffu, n == 4) && 4 * LPP * (strip + 1) <= L.mw && csize < (1u << 29);
+    const int xe = 4 * LPP * (strip + 1) - 1;                // the extra column
+    const int ry0 = seg * seg_rows, ry1 = min(oh, ry0 + seg_rows);
+    const int rx = 2 * (strip * LPP + ul);
+    const bool st0 = n > 0 && rx < ow, st1 = n > 0 && rx + 1 < ow;
     const DmPow pr = dm_pow_setup(lam);
-    float hp = -INFINITY;                                   // A row 2ry - 1 (none for ry = 0)
-    int cp = 0;
-    int ry = 0;
-    if (inside) {
-        // step ry reads child rows 2ry - 1 .. 2ry + 4: unchecked while they lie in the domain
-        stream_step<COMP, true>(w, 0, oh, hp, cp, pr, store, orow, arow, opitch);
-        for (ry = 2; 2 * ry + 4 < w.mh; ry += 2) stream_step<COMP, false>(w, ry, oh, hp, cp, pr, store, orow, arow, opitch);
+
+    // outputs: the patch's maps and the byte offset of (row ry, column rx) in the codes
+    char* ovals = reinterpret_cast<char*>(out + (size_t)p * oh * opitch);
+    unsigned char* ocodes = amax + (size_t)p * oh * opitch;
+    uint32_t oo = (uint32_t)ry0 * (uint32_t)opitch + (uint32_t)rx;
+    const uint32_t pitch4 = L.pitch4;
+    uint32_t off = (uint32_t)(2 * ry0 - 2) * pitch4 + (uint32_t)L.q0 * 4u;   // (row y - 1, column q0) of y = 2 ry0 - 1
+    LvRow r0;
+    if (any) {
+        const int y = 2 * ry0 - 1;
+        const float ex = lv_extra<COMP>(L, y, xe);
+        r0 = full && ry0 >= 2 && y + 1 < L.mh ? lv_row<COMP, true, LPP>(L, lv_load<true>(L, y, off), y, ex, 0)
+                                              : lv_row<COMP, false, LPP>(L, lv_load<false>(L, y, off), y, ex, 0);
     }
-    for (; ry < oh; ry += 2) stream_step<COMP, true>(w, ry, oh, hp, cp, pr, store, orow, arow, opitch);
+    off += pitch4;
+    for (int c0 = ry0; c0 < ry1; c0 += LPP / 2) {
+        __syncthreads();                                     // keeps the warps that share child rows together
+        if (!any) continue;
+        const float ex = lv_extra<COMP>(L, 2 * c0 + ul, xe);  // the extra column of the next LPP rows
+        const int c1 = min(ry1, c0 + LPP / 2);
+        for (int ry = c0; ry < c1; ry++) {
+            const int y = 2 * ry;
+            uint32_t k0, k1;
+            if (full && y >= 2 && y + 2 < L.mh) {
+                const LvKids v1 = lv_load<true>(L, y, off), v2 = lv_load<true>(L, y + 1, off + pitch4);
+                const LvRow r1 = lv_row<COMP, true, LPP>(L, v1, y, ex, y - 2 * c0);
+                const LvRow r2 = lv_row<COMP, true, LPP>(L, v2, y + 1, ex, y + 1 - 2 * c0);
+                const float b0 = lv_pool<0>(r0, r1, r2, k0), b1 = lv_pool<2>(r0, r1, r2, k1);
+                *reinterpret_cast<float2*>(ovals + (size_t)(4u * oo)) = dm_powf2(make_float2(b0, b1), pr);
+                *reinterpret_cast<unsigned short*>(ocodes + oo) = (unsigned short)(k0 | (k1 << 8));
+                r0 = r2;
+            } else {
+                const LvKids v1 = lv_load<false>(L, y, off), v2 = lv_load<false>(L, y + 1, off + pitch4);
+                const LvRow r1 = lv_row<COMP, false, LPP>(L, v1, y, ex, y - 2 * c0);
+                const LvRow r2 = lv_row<COMP, false, LPP>(L, v2, y + 1, ex, y + 1 - 2 * c0);
+                const float b0 = lv_pool<0>(r0, r1, r2, k0), b1 = lv_pool<2>(r0, r1, r2, k1);
+                // (lanes without an output evaluate the power of 1; a last odd column's
+                // partner lands in the row's padding)
+                const float2 pw = dm_powf2(make_float2(st0 ? b0 : 1.0f, st1 ? b1 : 1.0f), pr);
+                if (st0) {
+                    *reinterpret_cast<float2*>(ovals + (size_t)4 * oo) = pw;
+                    *reinterpret_cast<unsigned short*>(ocodes + oo) = (unsigned short)(k0 | (k1 << 8));
+                }
+                r0 = r2;
+            }
+            oo += (uint32_t)opitch;
+            off += 2u * pitch4;
+        }
+    }
 }
 
-template <bool COMP, bool APPROX = false>
-__global__ void __launch_bounds__(STREAM_WARPS * 32, 4) k_level_stream(DmGeom g, int l, const float* __restrict__ prev,
-                                                                   const unsigned char* __restrict__ vprev,
-                                                                   const unsigned char* __restrict__ vcur,
-                                                                   int bx_per_res, int by_per_res, float* __restrict__ out,
-                                                                   unsigned char* __restrict__ amax, float lam,
-                                                                   const int* __restrict__ proto_of, int n_maps) {
-    level_stream_body<COMP, APPROX>(g, l, prev, vprev, vcur, bx_per_res, by_per_res, out, amax, lam, proto_of, n_maps,
-                                    (long long)blockIdx.x);
+template <bool COMP, int LPP>
+__global__ void __launch_bounds__(LV_THREADS, 4)
+k_level_rows(DmGeom g, int l, const float* __restrict__ prev, const unsigned char* __restrict__ vprev, int nbx, int nby,
+             int seg_rows, float* __restrict__ out, unsigned char* __restrict__ amax, float lam,
+             const int* __restrict__ proto_of, int n_maps) {
+    level_rows_body<COMP, LPP>(g, l, prev, vprev, nbx, nby, seg_rows, out, amax, lam, proto_of, n_maps, blockIdx.x);
 }
 
 // Top level L: C_L = (mean of children)^lambda over the domain of level L.
@@ -676,19 +784,73 @@ cudaError_t launch_sweep(const DmGeom& g, int l, const CUtensorMap& tm, const dm
     return cudaGetLastError();
 }
 
-template <bool COMP, bool APPROX = false>
-cudaError_t launch_stream(const DmGeom& g, int l, const dm_pyramid& py, float lam, cudaStream_t st) {
-    const int S = l == 1 ? 1 : 1 << (l - 1);
-    const int bx_per_res = ((g.Lx + S - 1) / S + STREAM_BX - 1) / STREAM_BX;
-    const int by_per_res = ((g.Ly + S - 1) / S + STREAM_BY - 1) / STREAM_BY;
-    const int strips = (g.dw[l + 1] + STREAM_W - 1) / STREAM_W;
-    const long long blocks = (long long)strips * S * by_per_res * S * bx_per_res;
-    if (blocks <= 0) return cudaSuccess;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    k_level_stream<COMP, APPROX><<<(unsigned)blocks, STREAM_WARPS * 32, 0, st>>>(
-        g, l, py.pooled[l - 1], py.valid[l - 1], py.valid[l], bx_per_res, by_per_res, const_cast<float*>(py.pooled[l]),
-        const_cast<unsigned char*>(py.amax[l]), lam, APPROX ? py.proto_of : nullptr, py.n0_maps);
+// Launch shape of the row-streaming kernel at level l.
+struct LvShape {
+    int lpp, nbx, nby, seg_rows;     // lanes per unit, blocks of patches per residue, rows per segment
+    double fill;                     // share of the units' pooled columns that exist
+    long long blocks;
+};
+
+LvShape level_shape(const DmGeom& g, int l) {
+    LvShape s;
+    const int ow = g.dw[l + 1], oh = g.dh[l + 1], S = level_stride(l);
+    // lanes per unit: the least lanes per row, a unit's memory sectors past its edges
+    // counted as 4 lanes
+    s.lpp = 32;
+    double best = 1e30;
+    for (int lpp = 32; lpp >= 4; lpp /= 2) {
+        const double cost = (double)((ow + 2 * lpp - 1) / (2 * lpp)) * (lpp + 4);
+        if (cost < best) { best = cost; s.lpp = lpp; }
+    }
+    const int strips = (ow + 2 * s.lpp - 1) / (2 * s.lpp);
+    s.fill = (double)ow / (2.0 * s.lpp * strips);
+    const int px = LV_WX * (32 / s.lpp);                     // patches along x of a CTA
+    s.nbx = ((g.Lx + S - 1) / S + px - 1) / px;
+    s.nby = ((g.Ly + S - 1) / S + LV_WY - 1) / LV_WY;
+    // segments of about 32 rows of outputs (each costs one more row of averages, and
+    // a shorter one keeps more of the child rows that two rows of patches share in L2:
+    // whole columns 6.34, 64 rows 6.34, 32 rows 6.34, 16 rows 6.50 ms for the levels of
+    // 1024x436), shorter where the patches alone leave the GPU idle
+    const long long per_seg = (long long)S * s.nby * strips * ((S * s.nbx + LV_GROUP - 1) / LV_GROUP) * LV_GROUP;
+    const long long segs = std::max<long long>((oh + 31) / 32, std::min<long long>((oh + 2) / 3, (1216 + per_seg - 1) / per_seg));
+    s.seg_rows = (int)((oh + segs - 1) / segs);
+    s.blocks = (long long)((oh + s.seg_rows - 1) / s.seg_rows) * per_seg;
+    return s;
+}
+
+template <bool COMP, int LPP>
+cudaError_t launch_rows_lpp(const DmGeom& g, int l, const dm_pyramid& py, const LvShape& s, float lam, cudaStream_t st) {
+    static std::atomic<unsigned long long> l1_done{0};
+    const cudaError_t e = dm_prefer_l1(reinterpret_cast<const void*>(k_level_rows<COMP, LPP>), l1_done);
+    if (e != cudaSuccess) return e;
+    k_level_rows<COMP, LPP><<<(unsigned)s.blocks, LV_THREADS, 0, st>>>(
+        g, l, py.pooled[l - 1], py.valid[l - 1], s.nbx, s.nby, s.seg_rows, const_cast<float*>(py.pooled[l]),
+        const_cast<unsigned char*>(py.amax[l]), lam, l == 1 ? py.proto_of : nullptr, py.n0_maps);
     return cudaGetLastError();
+}
+
+template <bool COMP>
+cudaError_t launch_rows(const DmGeom& g, int l, const dm_pyramid& py, const LvShape& s, float lam, cudaStream_t st) {
+    if (s.blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    if (s.lpp == 32) return launch_rows_lpp<COMP, 32>(g, l, py, s, lam, st);
+    if (s.lpp == 16) return launch_rows_lpp<COMP, 16>(g, l, py, s, lam, st);
+    if (s.lpp == 8) return launch_rows_lpp<COMP, 8>(g, l, py, s, lam, st);
+    return launch_rows_lpp<COMP, 4>(g, l, py, s, lam, st);
+}
+
+// Which kernel takes level l: the row-streaming one where the tuned shape asks for it
+// (level_th = 0); for maps of at most 16 columns and for small images, where the tiled
+// kernel's per-patch pipeline is latency-bound; and for wider maps whose rows fill its
+// 64-column strips (or its one 32-column strip) to 88 %: it moves less through L1
+// and L2 than the tiled kernel, which has no such granularity.  A fault-injection run
+// takes the tiled kernel, which holds the bounded waits.  Measured (ncu, us, tiled /
+// row-streaming; columns of the stored map in front): 1024x436 256 5362 / 4487, 128
+// 1362 / 1137, 64 395 / 309, 32 117 / 113, 1242x375 311 (97 % filled) 6043 / 5484, 512x224
+// 128 370 / 311, 256x256 64 132 / 113; 640x480 160 (83 %) 2497 / 2806, 80 807 / 909, 20 80 / 115,
+// 1242x375 156 (81 %) 1535 / 1790; 130x70 33 41 / 29.
+bool level_streams(const DmGeom& g, int l, const DmTune& tune, const LvShape& s) {
+    const int ow = g.dw[l + 1];
+    return tune.level_th == 0 || ow <= 16 || g.npatch(l) <= 2048 || (s.fill >= 0.88 && (s.lpp == 32 || ow <= 32));
 }
 
 // ---------------------------------------------------------------------------
@@ -708,6 +870,7 @@ struct LvPair {
     unsigned char* amax;
     int* err;
     int a, b;                  // tiled: runs per residue; row-streaming: blocks per residue in x, y
+    int seg_rows;              // row-streaming: rows per segment
     long long first;           // first block of this pair in the launch
 };
 struct LvBatch {
@@ -730,12 +893,12 @@ __global__ void __launch_bounds__(level_threads<TH>()) k_level_sweep_b(const __g
                                                                (int)((long long)blockIdx.x - P.first));
 }
 
-template <bool COMP>
-__global__ void __launch_bounds__(STREAM_WARPS * 32, 4) k_level_stream_b(const __grid_constant__ LvBatch B, int l, float lam) {
+template <bool COMP, int LPP>
+__global__ void __launch_bounds__(LV_THREADS, 4) k_level_rows_b(const __grid_constant__ LvBatch B, int l, float lam) {
     const int j = lv_pair_of(B, blockIdx.x);
     const LvPair& P = B.p[j];
-    level_stream_body<COMP, false>(P.g, l, P.prev, P.vprev, P.vcur, P.a, P.b, P.out, P.amax, lam, nullptr, 0,
-                                   (long long)blockIdx.x - P.first);
+    level_rows_body<COMP, LPP>(P.g, l, P.prev, P.vprev, P.a, P.b, P.seg_rows, P.out, P.amax, lam, nullptr, 0,
+                               (unsigned)((long long)blockIdx.x - P.first));
 }
 
 __global__ void k_valid_b(const __grid_constant__ LvBatch B, int l) {
@@ -778,19 +941,9 @@ cudaError_t dm_launch_levels(const DmGeom& g, const dm_pyramid& py, float lam, i
     k_fill_u8<<<(n0 + 255) / 256, 256, 0, st>>>(const_cast<unsigned char*>(py.valid[0]), n0, 1);
     for (int l = 1; l <= g.L; l++) {
         k_valid<<<(np + 255) / 256, 256, 0, st>>>(g, l, py.valid[l - 1], const_cast<unsigned char*>(py.valid[l]));
-        // the row-streaming kernel: as the tuned shape, and always for the levels
-        // whose stored maps are at most 16 columns wide, where the tiled kernel's
-        // per-patch pipeline is latency-bound (1024x436: levels 5-7 take 0.18
-        // instead of 0.38 ms); a fault-injection run takes the tiled kernel,
-        // which holds the bounded waits
-        const bool stream = py.tune.level_th == 0 || g.dw[l + 1] <= 16;
-        if (l < g.L && stream && py.inject_wait == 0) {
-            const bool approx = l == 1 && py.proto_of != nullptr;
-            cudaError_t e;
-            if (approx)
-                e = py.compensated ? launch_stream<true, true>(g, l, py, lam, st) : launch_stream<false, true>(g, l, py, lam, st);
-            else
-                e = py.compensated ? launch_stream<true>(g, l, py, lam, st) : launch_stream<false>(g, l, py, lam, st);
+        const LvShape sh = l < g.L ? level_shape(g, l) : LvShape();
+        if (l < g.L && py.inject_wait == 0 && level_streams(g, l, py.tune, sh)) {
+            const cudaError_t e = py.compensated ? launch_rows<true>(g, l, py, sh, lam, st) : launch_rows<false>(g, l, py, sh, lam, st);
             if (e != cudaSuccess) return e;
         } else if (l < g.L) {
             // pooled maps of level l-1: [npatch(l-1)][dh[l]][pitch(l)] floats
@@ -897,8 +1050,9 @@ cudaError_t dm_launch_levels_batch(const dm_pyramid* const* pys, int n, float la
             }
         }
         // the pairs below their top: one launch per kernel shape in use.
-        // shape 0: row-streaming; 1 + 2 (rows 16 / 8 / 4 as 0 / 1 / 2) + (ring == 3): tiled
-        for (int shape = 0; shape < 7; shape++) {
+        // shape 1 + 2 (rows 16 / 8 / 4 as 0 / 1 / 2) + (ring == 3): tiled; 7 .. 10:
+        // row-streaming with units of 32, 16, 8 and 4 lanes
+        for (int shape = 1; shape < 11; shape++) {
             LvBatch B;
             memset(&B, 0, sizeof(B));
             long long blocks = 0;
@@ -906,19 +1060,20 @@ cudaError_t dm_launch_levels_batch(const dm_pyramid* const* pys, int n, float la
                 const dm_pyramid& py = *pys[j];
                 const DmGeom& g = py.g;
                 if (l >= g.L) continue;
-                const bool stream = py.tune.level_th == 0 || g.dw[l + 1] <= 16;
+                const LvShape sh = level_shape(g, l);
+                const bool stream = level_streams(g, l, py.tune, sh);
                 const int th = py.tune.level_th == 8 || py.tune.level_th == 4 ? py.tune.level_th : 16;
                 const int nr = py.tune.level_ring == 3 ? 3 : 2;
-                const int my = stream ? 0 : 1 + 2 * (th == 16 ? 0 : (th == 8 ? 1 : 2)) + (nr == 3);
+                const int my = stream ? (sh.lpp == 32 ? 7 : sh.lpp == 16 ? 8 : sh.lpp == 8 ? 9 : 10) : 1 + 2 * (th == 16 ? 0 : (th == 8 ? 1 : 2)) + (nr == 3);
                 if (my != shape) continue;
                 LvPair q = base_pair(j, l);
                 const int S = l == 1 ? 1 : 1 << (l - 1);
                 long long items;
                 if (stream) {
-                    q.a = ((g.Lx + S - 1) / S + STREAM_BX - 1) / STREAM_BX;
-                    q.b = ((g.Ly + S - 1) / S + STREAM_BY - 1) / STREAM_BY;
-                    const int strips = (g.dw[l + 1] + STREAM_W - 1) / STREAM_W;
-                    items = (long long)strips * S * q.b * S * q.a;
+                    q.a = sh.nbx;
+                    q.b = sh.nby;
+                    q.seg_rows = sh.seg_rows;
+                    items = sh.blocks;
                 } else {
                     const cuuint64_t dims[3] = {(cuuint64_t)g.dw[l], (cuuint64_t)g.dh[l], (cuuint64_t)g.npatch(l - 1)};
                     const cuuint64_t strides[2] = {(cuuint64_t)g.pitch(l) * 4, (cuuint64_t)g.psize(l) * 4};
@@ -938,9 +1093,17 @@ cudaError_t dm_launch_levels_batch(const dm_pyramid* const* pys, int n, float la
             if (B.n == 0 || blocks == 0) continue;
             if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
             cudaError_t e = cudaSuccess;
-            if (shape == 0) {
-                if (comp) k_level_stream_b<true><<<(unsigned)blocks, STREAM_WARPS * 32, 0, st>>>(B, l, lam);
-                else k_level_stream_b<false><<<(unsigned)blocks, STREAM_WARPS * 32, 0, st>>>(B, l, lam);
+            if (shape >= 7) {
+                static std::atomic<unsigned long long> l1_done[8];
+                auto go = [&](auto kern) -> cudaError_t {
+                    const cudaError_t el = dm_prefer_l1(reinterpret_cast<const void*>(kern), l1_done[2 * (shape - 7) + comp]);
+                    if (el == cudaSuccess) kern<<<(unsigned)blocks, LV_THREADS, 0, st>>>(B, l, lam);
+                    return el;
+                };
+                if (shape == 7) e = comp ? go(k_level_rows_b<true, 32>) : go(k_level_rows_b<false, 32>);
+                else if (shape == 8) e = comp ? go(k_level_rows_b<true, 16>) : go(k_level_rows_b<false, 16>);
+                else if (shape == 9) e = comp ? go(k_level_rows_b<true, 8>) : go(k_level_rows_b<false, 8>);
+                else e = comp ? go(k_level_rows_b<true, 4>) : go(k_level_rows_b<false, 4>);
             } else {
                 auto launch = [&](auto kern, int TH, int NR) -> cudaError_t {
                     const int kidf = (((2 * TH + 1) * KW + 31) / 32) * 32;     // LevelTile<TH>::KIDF
