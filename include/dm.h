@@ -489,14 +489,15 @@ dm_status dm_autotune_batch(dm_ctx* ctx, int n, const dm_pair* pairs, void* d_ws
  * kernels on the given pair and keeps, for pairs of exactly these sizes in
  * this context, the fastest of each:
  *   chosen[0]  M-tiles (128 patches each) per work unit of the tensor-core
- *              level-0 kernel (the work unit is one N-tile x that many
- *              M-tiles; candidates split the patches into 1, 2, 3, 4, 6 or 8
- *              chunks; unused by DM_FP32);
+ *              level-0 kernel, at most (the work unit is a pair of N-tiles x
+ *              that many M-tiles, fewer where that fills the GPU's last round of
+ *              units better; candidates split the patches into 1, 2, 3, 4, 6
+ *              or 8 chunks; unused by DM_FP32);
  *   chosen[1]  level kernel: pooled rows per CTA tile of the tiled kernel (16,
  *              8 or 4, on 8, 4 or 2 warps), or 0 for the row-streaming kernel
- *              (one warp per patch and 31-column strip, no shared memory);
- *              levels whose stored maps are at most 16 columns wide always
- *              take the latter;
+ *              (registers only, strips of 64 columns) at every level; levels
+ *              whose stored maps are at most 16 columns wide or fill its strips,
+ *              and small images, always take the latter;
  *   chosen[2]  CTAs per SM of the backtracking expansion kernels (2..32);
  *   chosen[3]  child-window columns in the level kernel's ring (3 or 2).
  * Every candidate computes identical results; only the time differs.  Each

@@ -12,11 +12,10 @@
 //      matrix; 18 core matrices along K per 8-row group, 2304 bytes), so one
 //      36,864-byte bulk copy (cp.async.bulk, TMA engine) moves a tile to
 //      shared memory.
-//   B: the implicit im2col of I' for one N-tile of 33 x 7 positions (231 of
-//      the 240 rows of the MMA), built in shared memory by all warps in the
+//   B: the implicit im2col of I' for two N-tiles side by side, 33 x 7 positions each
+//      (231 of the 240 rows of the MMA), built in shared memory by all warps in the
 //      same layout and kept resident while the CTA sweeps a chunk of M-tiles.
-//   D: 128 lanes x 240 FP32 columns of TMEM; two accumulators (columns 0 and
-//      256) let the epilogue drain one tile while the next is multiplied.
+//   D: 128 lanes x 240 FP32 columns of TMEM per N-tile (columns 0 and 256).
 // Pooling geometry: the N-tile's positions are x = 2 rx0 - 1 + lx (lx < 33),
 // y = 2 ry0 - 1 + ly (ly < 7); they cover the 3x3 windows of the 16 x 3
 // pooled outputs (rx0 + k, ry0 + j), centre lx = 2k + 1, ly = 2j + 1.
@@ -24,21 +23,30 @@
 // Output path.  P_0 is stored patch-major ([patch][row][pitch]), so the 16
 // pooled values of one tile row of one patch are 64 contiguous bytes (16 for
 // the argmax codes).  Plain per-thread stores scatter each warp store over 32
-// patches (32 sectors per instruction) and saturate L1.  Instead the
-// epilogue writes each tile's 128 x 3 x 16 outputs into a shared-memory
-// staging buffer (double-buffered) and one thread hands it to the TMA engine
-// with two 3-D tensor stores (values, codes); the tensor maps clip rows and
-// columns outside the maps and patches past the last one.
+// patches (32 sectors per instruction) and saturate L1.  Instead the epilogue
+// stages each tile's 128 x 3 x 16 values, and the pair's 128 x 3 x 32 codes, in
+// shared memory and one thread hands them to the TMA engine with 3-D tensor
+// stores; the tensor maps clip rows and columns outside the maps and patches past
+// the last one.  The pair is there for the codes: the 16-byte rows of a single
+// N-tile are halves of a memory sector, and two CTAs that fill the halves at
+// different times cost a read-modify-write of DRAM (without the store of the codes
+// the single form took 5.0 instead of 6.0 ms in BF16 at 1024x436 and 4.8 instead of
+// 9.9 ms in FP8 with two chunks of M-tiles); rows of 32 codes are whole sectors.
 //
-// Warp roles (576 threads, one CTA per SM, persistent over work units
-// (N-tile, M-chunk)): warp 0 issues the bulk copies of A (2-stage ring),
-// warp 1 allocates TMEM and one lane issues the MMAs and commits, warps 2-17
-// drain the accumulators: four warps per TMEM lane quadrant, each owning four
-// of the sixteen pooled columns (C0 columns 8w'..8w'+8) over the three pooled
-// rows: 14 tcgen05.ld in three batches of rows (each batch in flight while the
-// rows before it are pooled), pool on order-preserving keys that carry the
-// position (first maximum in scan order), release the accumulator after the last batch,
-// raise to lambda (MUFU-based power), stage, store through TMA.
+// Warp roles (608 threads, one CTA per SM, persistent over work units (pair of
+// N-tiles, M-chunk)): warp 0 issues the bulk copies of A, warp 1 allocates TMEM and
+// one lane issues the MMAs of both N-tiles and commits, warps 2-17 drain the
+// accumulators, warp 18 issues the stores.  The draining warps form two groups of
+// eight, one per N-tile: four TMEM lane quadrants x two halves of eight pooled columns,
+// each half in two parts of four (C0 columns 8w'..8w'+8) over the three pooled rows:
+// 14 tcgen05.ld per part in three batches of rows (each batch in flight while the rows
+// before it are pooled), pool on order-preserving keys that carry the position (first
+// maximum in scan order), raise to lambda (MUFU-based power), stage.
+// What bounds it: the draining, by latency at four warps per scheduler (27 instructions
+// per output at 45 % issue); with a single K step instead of nine it would take 4.9 ms,
+// with stores that nothing waits for 5.3, of 5.38 ms (1024x436, BF16; 3.0 TB/s written).
+// 1024x436: BF16 6.05 -> 5.38 ms, FP8 9.9 -> 5.16; 640x480 BF16 3.06 -> 2.44; 1242x375 FP8
+// 10.8 -> 6.3.
 // FP8 form: the same kernel with E4M3 operands (tcgen05.mma kind::f8f6f4,
 // K padded 144 -> 160, five MMAs of K = 32).  Each patch vector is scaled by a
 // power of two that brings its largest entry into (224, 448] (E4M3's top
@@ -51,9 +59,12 @@
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
+#include <algorithm>
+
 #include "dm_internal.cuh"
 
 #include <memory>
+#include <type_traits>
 
 namespace {
 
@@ -61,12 +72,17 @@ constexpr int BM = 128;                       // patches per M-tile (TMEM lanes)
 constexpr int KD = 144;                       // 4 x 4 x 9
 constexpr int CX = 33, CY = 7;                // C0 positions per N-tile
 constexpr int BN = 240;                       // CX * CY = 231, padded to a multiple of 16
+constexpr int BROWS = 232;                    // operand rows kept per N-tile; the MMA reads 240: the last 8 are
+                                              // whatever follows in shared memory, for columns nothing reads
 constexpr int PX = 16, PY = 3;                // pooled outputs per N-tile
+constexpr int SX = 2 * PX;                    // pooled columns of a pair of N-tiles
 constexpr int EPI_WARPS = 16;
-constexpr int EPI_THREADS = 32 * EPI_WARPS;
-constexpr int THREADS = 64 + EPI_THREADS;
-constexpr int OUT_F = BM * PY * PX * 4;       // 24576: staged values of one tile
-constexpr int OUT_C = BM * PY * PX;           // 6144: staged argmax codes of one tile
+constexpr int GROUP_THREADS = 16 * EPI_WARPS; // draining threads of one accumulator (half of the draining warps)
+constexpr int STORE_WARP = 2 + EPI_WARPS;
+constexpr int THREADS = 32 * (STORE_WARP + 1);
+constexpr int WIN_ROWS = CY + 3, WIN_COLS = (2 * PX + CX + 3) * 9;   // field window of a pair (pixels x 9)
+constexpr int OUT_F = BM * PY * PX * 4;       // 24576: staged values of one N-tile's tile
+constexpr int OUT_C = BM * PY * SX;           // 12288: staged argmax codes of a pair's tile
 constexpr long long WAIT_CYCLES = 4000000000LL;     // ~2 s at 2 GHz
 
 enum { FMT_BF16 = 0, FMT_E4M3 = 1 };
@@ -78,6 +94,7 @@ template <int FMT>
 struct Fmt {
     static constexpr int KP = FMT == FMT_BF16 ? 144 : 160;
     static constexpr int ESZ = FMT == FMT_BF16 ? 2 : 1;
+    using Elem = std::conditional_t<FMT == FMT_BF16, unsigned short, unsigned char>;
     static constexpr int KSTEP = FMT == FMT_BF16 ? 16 : 32;
     static constexpr int KSTEPS = KP / KSTEP;
     static constexpr int ROWB = KP * ESZ;              // bytes per operand row
@@ -85,18 +102,21 @@ struct Fmt {
     static constexpr int EPC = 16 / ESZ;               // elements per 16-byte chunk
     static constexpr int GROUP = CHUNKS * 128;         // bytes per 8-row group
     static constexpr int A_TILE = BM * ROWB;
-    static constexpr int B_TILE = BN * ROWB;
-    static constexpr int STAGES = FMT == FMT_BF16 ? 2 : 3;
-    static constexpr int OFF_B = 0;
-    static constexpr int OFF_A = ((B_TILE + 1023) / 1024) * 1024;
-    static constexpr int OFF_F = ((OFF_A + STAGES * A_TILE + 1023) / 1024) * 1024;
+    static constexpr int B_TILE = BROWS * ROWB;
+    static constexpr int STAGES = FMT == FMT_BF16 ? 1 : 2;
+    static constexpr int OFF_F = 0;                    // (swizzled buffers: 512- and 256-byte aligned)
     static constexpr int OFF_C = OFF_F + 2 * OUT_F;
-    static constexpr int OFF_BAR = OFF_C + 2 * OUT_C;
+    static constexpr int OFF_B = OFF_C + OUT_C;
+    static constexpr int OFF_A = OFF_B + 2 * B_TILE;
+    static constexpr int OFF_BAR = OFF_A + STAGES * A_TILE;
     static constexpr size_t SMEM = (size_t)OFF_BAR + 256;
     static constexpr uint32_t IDESC = (1u << 4) | (FMT == FMT_BF16 ? ((1u << 7) | (1u << 10)) : 0u) |
                                       ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 };
 static_assert(Fmt<FMT_BF16>::SMEM <= 232448 && Fmt<FMT_E4M3>::SMEM <= 232448, "shared memory");
+static_assert(Fmt<FMT_BF16>::OFF_A % 128 == 0 && Fmt<FMT_E4M3>::OFF_A % 128 == 0 && Fmt<FMT_BF16>::OFF_C % 1024 == 0, "alignment");
+static_assert(WIN_ROWS * WIN_COLS * 2 <= 2 * OUT_F && KD % 16 == 0 && (2 * PX + CX + 3) == 68, "window");
+static_assert((BN - BROWS) * Fmt<FMT_BF16>::ROWB <= Fmt<FMT_BF16>::A_TILE, "the second operand tile's last rows stay in shared memory");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -141,8 +161,6 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-
-__device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, %0;" :: "n"(EPI_THREADS) : "memory"); }
 
 // Pack the patch vectors of I into BF16 M-tiles (zero rows past the last patch).
 // Rows: image 1's atomic patches (from d1), or the n0 vectors of amat
@@ -235,7 +253,8 @@ __global__ void k_pack_a8(DmGeom g, const float* __restrict__ d1, unsigned char*
 struct EpiArgs {
     uint32_t taddr;     // TMEM address of this warp's lane quadrant, column 0
     int row;            // accumulator row (patch within the M-tile)
-    int part;           // pooled columns 4*part .. 4*part+3
+    int half;           // pooled columns 8*half .. 8*half+7 of the N-tile, two parts of 4
+    int tile;           // 0 or 1: the N-tile (and accumulator) of the pair
     int cx0, cy0, W2, H2;
     float lam;
     bool interior;      // every C0 position of the N-tile lies inside I'
@@ -324,9 +343,9 @@ __device__ __forceinline__ float lam_log2_pow2(float x, float lam) {
 
 // Vertical step for pooled row y (C0 rows 2y, 2y+1, 2y+2 = m_y -1, 0, +1): the
 // key maximum, its code 3 (row - 2y) + (c - 2k) from the low bits, the power,
-// and the staging of the 4 values and codes.
-__device__ __forceinline__ void pool_out(const EpiArgs& e, int y, float lc, const float (&h)[CY][4],
-                                         float* stage_f, unsigned char* stage_c) {
+// and the staging of the 4 values; returns the 4 codes.
+__device__ __forceinline__ uint32_t pool_out(const EpiArgs& e, int part, int y, float lc, const float (&h)[CY][4],
+                                             float* stage_f) {
     float f[4];
     uint32_t mb[4];
 #pragma unroll
@@ -345,61 +364,91 @@ __device__ __forceinline__ void pool_out(const EpiArgs& e, int y, float lc, cons
     asm("prmt.b32 %0, %1, %2, 0x5410;" : "=r"(lo) : "r"(lo01), "r"(lo23));
     const uint32_t cst = (uint32_t)(31 - 6 * y) * 0x01010101u - 0x06040200u;   // bytes 31 - 6y - 2k
     const uint32_t codes = cst - (lo & 0x1F1F1F1Fu);
-    // staging layout = the TMA box [patch][row][16 columns].  The values' box
-    // rows (64 bytes, four 16-byte chunks) are staged with the tensor map's
-    // 64-byte swizzle: the 16-byte chunk index (shared address bits 4-5) is
-    // XORed with address bits 7-8 of the row.  Lanes hold consecutive patches,
-    // box rows 3 apart, so without it the 16-byte stores of a quarter warp
-    // would hit the same four banks four times.
+    // staging layout = the TMA box [patch][row][16 columns] of the N-tile.  Its rows
+    // (64 bytes, four 16-byte chunks) are staged with the tensor map's 64-byte
+    // swizzle: the 16-byte chunk index (shared address bits 4-5) is XORed with address
+    // bits 7-8 of the row.  Lanes hold consecutive patches, box rows 3 apart, so
+    // without it the 16-byte stores of a quarter warp would hit the same four banks
+    // four times.
     const int R = e.row * PY + y;
     const uint32_t row_addr = smem_u32(stage_f) + (uint32_t)R * (PX * 4);
-    const int chunk = e.part ^ (int)((row_addr >> 7) & 3u);
+    const int chunk = part ^ (int)((row_addr >> 7) & 3u);
     *reinterpret_cast<float4*>(stage_f + R * PX + 4 * chunk) = make_float4(f[0], f[1], f[2], f[3]);
-    *reinterpret_cast<uint32_t*>(stage_c + R * PX + 4 * e.part) = codes;
+    return codes;
 }
 
-// Pool this thread's 4 x 3 outputs of one accumulator, release the
-// accumulator, and write the powered values and codes to the staging buffer.
-// `mult` turns an accumulator value into C0 (1/16, times the inverse operand
-// scales of the FP8 form; positive, so pooling on raw accumulators is exact).
-// The seven accumulator rows are read in three batches (rows 0-2, 3-4, 5-6):
-// each batch's loads are in flight while the rows before it are pooled, and
-// pooled row y is finished as soon as its C0 rows 2y .. 2y+2 are in.
-__device__ __forceinline__ void epilogue_tile(const EpiArgs& e, uint32_t b, uint32_t bar_empty, float mult,
-                                              float* stage_f, unsigned char* stage_c) {
+// Stage the codes of one part's three pooled rows: the box [patch][row][32 columns] of
+// the pair, the N-tiles side by side, its 32-byte rows with the 32-byte swizzle (the
+// 16-byte chunk XORed with bit 2 of the row).
+__device__ __forceinline__ void stage_codes(const EpiArgs& e, int part, const uint32_t (&c)[PY], unsigned char* stage_c) {
+#pragma unroll
+    for (int y = 0; y < PY; y++) {
+        const int R = e.row * PY + y;
+        *reinterpret_cast<uint32_t*>(stage_c + R * SX + 16 * (e.tile ^ ((R >> 2) & 1)) + 4 * part) = c[y];
+    }
+}
+
+// Pool this thread's 8 x 3 outputs of one accumulator in two parts of 4 columns,
+// release the accumulator, and write the powered values and codes to the staging
+// buffers once `values_free` and `codes_free` say that the stores before have read
+// them (the codes wait in registers until the end of their part: their buffer is
+// shared by both groups, so it is free later).  `mult` turns an
+// accumulator value into C0 (1/16, times the inverse operand scales of the FP8 form;
+// positive, so pooling on raw accumulators is exact).  The seven accumulator rows of
+// a part are read in three batches (rows 0-2, 3-4, 5-6): each batch's loads are in
+// flight while the rows before it are pooled (the second part's first batch during
+// the end of the first part), and pooled row y is finished as soon as its C0 rows
+// 2y .. 2y+2 are in.
+template <class VFree, class CFree>
+__device__ __forceinline__ void epilogue_tile(const EpiArgs& e, uint32_t bar_empty, float mult,
+                                              float* stage_f, unsigned char* stage_c, VFree values_free, CFree codes_free) {
     const float lc = lam_log2_pow2(mult, e.lam);
     uint32_t r[CY][9];
-    float h[CY][4];
-    const uint32_t taddr = e.taddr + b * 256 + 8 * e.part;
-    const int tx0 = e.cx0 + 8 * e.part;
+    const uint32_t tbase = e.taddr + 16 * e.half;
 #pragma unroll
-    for (int ly = 0; ly < 3; ly++) tmem_row(taddr, ly, r[ly]);
-    tmem_wait();
+    for (int ly = 0; ly < 3; ly++) tmem_row(tbase, ly, r[ly]);
 #pragma unroll
-    for (int ly = 0; ly < 3; ly++) tmem_row_ready(r[ly]);
+    for (int q = 0; q < 2; q++) {
+        float h[CY][4];
+        uint32_t codes[PY];
+        const int part = 2 * e.half + q;
+        const uint32_t taddr = tbase + 8 * q;
+        const int tx0 = e.cx0 + 8 * part;
+        tmem_wait();
 #pragma unroll
-    for (int ly = 3; ly < 5; ly++) tmem_row(taddr, ly, r[ly]);
-    pool_row<0>(e, tx0, r[0], h[0]);
-    pool_row<1>(e, tx0, r[1], h[1]);
-    pool_row<2>(e, tx0, r[2], h[2]);
-    pool_out(e, 0, lc, h, stage_f, stage_c);
-    tmem_wait();
+        for (int ly = 0; ly < 3; ly++) tmem_row_ready(r[ly]);
 #pragma unroll
-    for (int ly = 3; ly < 5; ly++) tmem_row_ready(r[ly]);
+        for (int ly = 3; ly < 5; ly++) tmem_row(taddr, ly, r[ly]);
+        pool_row<0>(e, tx0, r[0], h[0]);
+        pool_row<1>(e, tx0, r[1], h[1]);
+        pool_row<2>(e, tx0, r[2], h[2]);
+        if (q == 0) values_free();
+        codes[0] = pool_out(e, part, 0, lc, h, stage_f);
+        tmem_wait();
 #pragma unroll
-    for (int ly = 5; ly < 7; ly++) tmem_row(taddr, ly, r[ly]);
-    pool_row<3>(e, tx0, r[3], h[3]);
-    pool_row<4>(e, tx0, r[4], h[4]);
-    pool_out(e, 1, lc, h, stage_f, stage_c);
-    tmem_wait();
+        for (int ly = 3; ly < 5; ly++) tmem_row_ready(r[ly]);
 #pragma unroll
-    for (int ly = 5; ly < 7; ly++) tmem_row_ready(r[ly]);
-    // every load of this accumulator is complete: hand it back to the MMA warp
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    mbar_arrive(bar_empty);
-    pool_row<5>(e, tx0, r[5], h[5]);
-    pool_row<6>(e, tx0, r[6], h[6]);
-    pool_out(e, 2, lc, h, stage_f, stage_c);
+        for (int ly = 5; ly < 7; ly++) tmem_row(taddr, ly, r[ly]);
+        pool_row<3>(e, tx0, r[3], h[3]);
+        pool_row<4>(e, tx0, r[4], h[4]);
+        codes[1] = pool_out(e, part, 1, lc, h, stage_f);
+        tmem_wait();
+#pragma unroll
+        for (int ly = 5; ly < 7; ly++) tmem_row_ready(r[ly]);
+        if (q == 0) {
+#pragma unroll
+            for (int ly = 0; ly < 3; ly++) tmem_row(taddr + 8, ly, r[ly]);
+        } else {
+            // every load of this accumulator is complete: hand it back to the MMA warp
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mbar_arrive(bar_empty);
+        }
+        pool_row<5>(e, tx0, r[5], h[5]);
+        pool_row<6>(e, tx0, r[6], h[6]);
+        codes[2] = pool_out(e, part, 2, lc, h, stage_f);
+        if (q == 0) codes_free();
+        stage_codes(e, part, codes, stage_c);
+    }
 }
 
 // Per-pair arguments of the level-0 kernel.  One launch serves one pair, or
@@ -434,10 +483,13 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
     float* sF = reinterpret_cast<float*>(smem + F::OFF_F);
     unsigned char* sC = smem + F::OFF_C;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + F::OFF_BAR);
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 2 * F::STAGES + 4);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 2 * F::STAGES + 9);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
     const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + F::STAGES);
     const uint32_t bar_acc_full = smem_u32(bars + 2 * F::STAGES), bar_acc_empty = smem_u32(bars + 2 * F::STAGES + 2);
+    // group b has staged its tile; the stores have read group b's values, the codes
+    const uint32_t bar_staged = smem_u32(bars + 2 * F::STAGES + 4), bar_vfree = smem_u32(bars + 2 * F::STAGES + 6);
+    const uint32_t bar_cfree = smem_u32(bars + 2 * F::STAGES + 8);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
@@ -447,8 +499,11 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
         }
         for (int b = 0; b < 2; b++) {
             mbar_init(bar_acc_full + 8 * b, 1);
-            mbar_init(bar_acc_empty + 8 * b, EPI_THREADS);
+            mbar_init(bar_acc_empty + 8 * b, GROUP_THREADS);
+            mbar_init(bar_staged + 8 * b, EPI_WARPS / 2);
+            mbar_init(bar_vfree + 8 * b, 1);
         }
+        mbar_init(bar_cfree, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -460,8 +515,8 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_holder;
 
-    uint32_t a_it = 0, acc_it = 0;
-    const bool store_leader = (warp == 2 && lane == 0);
+    // tiles so far: A tiles (and stores), and those of accumulator 1
+    uint32_t a_it = 0, acc1_it = 0;
 
     for (int gu = blockIdx.x; gu < B.total; gu += gridDim.x) {
         int pj = 0;
@@ -472,38 +527,50 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
         const float* __restrict__ d2 = P.d2;
         int* __restrict__ err = P.err;
         const int W2 = P.g.W2, H2 = P.g.H2, mw = P.g.dw[1];
-        const int tiles_x = (mw + PX - 1) / PX;
+        const int pairs_x = (mw + SX - 1) / SX;
         const int mchunks = (P.n_mtiles + P.m_chunk - 1) / P.m_chunk;
         // image-2 operand scale of the FP8 form (power of two from the field's maximum)
         const float s_b = FMT == FMT_E4M3 ? e4m3_scale(__uint_as_float(*P.bmax)) : 1.0f;
         const int unit = gu - P.first;
         const int m_chunk = P.m_chunk, n_mtiles = P.n_mtiles;
-        const int ntile = unit / mchunks, mc = unit % mchunks;
+        const int npairs = P.units / mchunks, pair = unit % npairs, mc = unit / npairs;
         const int m0 = mc * m_chunk, m1 = min(n_mtiles, m0 + m_chunk), nt = m1 - m0;
-        const int rx0 = (ntile % tiles_x) * PX, ry0 = (ntile / tiles_x) * PY;
+        const int rx0 = (pair % pairs_x) * SX, ry0 = (pair / pairs_x) * PY;
         const int cx0 = 2 * rx0 - 1, cy0 = 2 * ry0 - 1;
+        const bool two = rx0 + PX < mw;          // the pair's second N-tile holds pooled columns
 
-        // B: implicit im2col of I' for this N-tile (zero outside I', past K = 144
-        // and in rows 231..239), one 16-byte core-matrix row per item
-        for (int ch = tid; ch < BN * F::CHUNKS; ch += THREADS) {
-            const int n = ch / F::CHUNKS, kc = ch % F::CHUNKS;
+        // B: implicit im2col of I' for both N-tiles.  The pair's window of the field (10 rows
+        // of 68 pixels, zero outside I') is converted to the operand type once, into the
+        // staging buffers, which hold no tile between units; then every 16-byte
+        // core-matrix row is gathered from there: along k a window row (dy fixed) is 36
+        // consecutive elements, and an item crosses at most one such boundary.  (Gathered
+        // from global memory this took as long as 8 tiles of 128 patches.)
+        using E = typename F::Elem;
+        E* win = reinterpret_cast<E*>(smem + F::OFF_F);
+        for (int i = tid; i < WIN_ROWS * WIN_COLS; i += THREADS) {
+            const int row = i / WIN_COLS, q = i - row * WIN_COLS;
+            const int x9 = (cx0 - 2) * 9 + q, y = cy0 - 2 + row;
+            const float f = x9 >= 0 && x9 < W2 * 9 && y >= 0 && y < H2 ? __ldg(d2 + (long long)y * W2 * 9 + x9) : 0.0f;
+            if constexpr (FMT == FMT_BF16) win[i] = __bfloat16_as_ushort(__float2bfloat16_rn(f));
+            else win[i] = __nv_cvt_float_to_fp8(f * s_b, __NV_SATFINITE, __NV_E4M3);
+        }
+        __syncthreads();
+        for (int ch = tid; ch < (two ? 2 : 1) * BROWS * F::CHUNKS; ch += THREADS) {
+            const int nn = ch / F::CHUNKS, kc = ch % F::CHUNKS;
+            const int g = nn >= BROWS, n = nn - g * BROWS;
             const int lx = n % CX, ly = n / CX;
-            const int tx = cx0 + lx, ty = cy0 + ly;
+            const int k0 = kc * F::EPC, dy0 = k0 / 36, r0 = k0 - 36 * dy0;
+            const E* src = win + (ly + dy0) * WIN_COLS + (2 * PX * g + lx) * 9 + r0;
             uint32_t w[4] = {0u, 0u, 0u, 0u};
+            if (n < CX * CY && k0 < KD) {                    // (KD is a multiple of the elements of an item)
 #pragma unroll
-            for (int e = 0; e < F::EPC; e++) {
-                const int k = kc * F::EPC + e;
-                const int dy = k / 36, dx = (k / 9) % 4, c = k % 9;
-                const int x = tx - 2 + dx, y = ty - 2 + dy;
-                const float f = (k < KD && n < CX * CY && x >= 0 && y >= 0 && x < W2 && y < H2)
-                                    ? __ldg(d2 + ((long long)y * W2 + x) * 9 + c) : 0.0f;
-                if (FMT == FMT_BF16) {
-                    w[e >> 1] |= (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(f)) << (16 * (e & 1));
-                } else {
-                    w[e >> 2] |= (uint32_t)__nv_cvt_float_to_fp8(f * s_b, __NV_SATFINITE, __NV_E4M3) << (8 * (e & 3));
+                for (int e = 0; e < F::EPC; e++) {
+                    const uint32_t v = src[r0 + e >= 36 ? e + WIN_COLS - 36 : e];
+                    w[e * F::ESZ >> 2] |= v << (8 * (e * F::ESZ & 3));
                 }
             }
-            *reinterpret_cast<uint4*>(sB + (n >> 3) * F::GROUP + kc * 128 + (n & 7) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4*>(sB + g * F::B_TILE + (n >> 3) * F::GROUP + kc * 128 + (n & 7) * 16) =
+                make_uint4(w[0], w[1], w[2], w[3]);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
@@ -521,96 +588,130 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
             }
         } else if (warp == 1) {
             if (lane == 0) {
-                for (int j = 0; j < nt; j++) {
+                bool ok = true;
+                for (int j = 0; ok && j < nt; j++) {
                     const uint32_t it = a_it + j, s = it % F::STAGES, ph = (it / F::STAGES) & 1;
-                    const uint32_t ai = acc_it + j, b = ai & 1, aph = (ai >> 1) & 1;
-                    if (!mbar_wait(bar_full + 8 * s, ph, abort_flag, err)) break;
-                    if (!mbar_wait(bar_acc_empty + 8 * b, aph ^ 1, abort_flag, err)) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t d_tmem = tmem + b * 256;
-                    const uint32_t a_base = smem_u32(sA + s * F::A_TILE), b_base = smem_u32(sB);
+                    ok = mbar_wait(bar_full + 8 * s, ph, abort_flag, err);
+                    for (int b = 0; ok && b < (two ? 2 : 1); b++) {
+                        const uint32_t aph = (b ? acc1_it + j : it) & 1;
+                        ok = mbar_wait(bar_acc_empty + 8 * b, aph ^ 1, abort_flag, err);
+                        if (!ok) break;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t d_tmem = tmem + b * 256;
+                        const uint32_t a_base = smem_u32(sA + s * F::A_TILE), b_base = smem_u32(sB + b * F::B_TILE);
 #pragma unroll
-                    for (int k = 0; k < F::KSTEPS; k++) {
-                        const uint64_t ad = make_desc(a_base + k * 256, F::GROUP), bd = make_desc(b_base + k * 256, F::GROUP);
-                        const uint32_t acc = k > 0;
-                        if (FMT == FMT_BF16)
-                            asm volatile("{.reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;}"
-                                         :: "r"(d_tmem), "l"(ad), "l"(bd), "r"(F::IDESC), "r"(acc) : "memory");
-                        else
-                            asm volatile("{.reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;}"
-                                         :: "r"(d_tmem), "l"(ad), "l"(bd), "r"(F::IDESC), "r"(acc) : "memory");
+                        for (int k = 0; k < F::KSTEPS; k++) {
+                            const uint64_t ad = make_desc(a_base + k * 256, F::GROUP), bd = make_desc(b_base + k * 256, F::GROUP);
+                            const uint32_t acc = k > 0;
+                            if (FMT == FMT_BF16)
+                                asm volatile("{.reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;}"
+                                             :: "r"(d_tmem), "l"(ad), "l"(bd), "r"(F::IDESC), "r"(acc) : "memory");
+                            else
+                                asm volatile("{.reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;}"
+                                             :: "r"(d_tmem), "l"(ad), "l"(bd), "r"(F::IDESC), "r"(acc) : "memory");
+                        }
+                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar_acc_full + 8 * b) : "memory");
                     }
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar_empty + 8 * s) : "memory");
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar_acc_full + 8 * b) : "memory");
+                    if (ok)
+                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar_empty + 8 * s) : "memory");
+                }
+            }
+        } else if (warp == STORE_WARP) {
+            // one thread hands the staged tiles to the TMA engine -- the values of each group
+            // by themselves, as soon as they are there (rows of 64 bytes), the codes of both
+            // together, as rows of 32 bytes: a 16-byte row is half a memory sector, and two
+            // CTAs filling the halves of one cost up to 4 ms of read-modify-write at 1024x436
+            // -- and passes on that the stores have read the buffers
+            if (lane == 0) {
+                for (int j = 0; j < nt; j++) {
+                    const uint32_t ph = (a_it + j) & 1;
+                    const int z = (m0 + j) * BM;
+                    for (int b = 0; b < 2; b++) {
+                        if (mbar_wait(bar_staged + 8 * b, ph, abort_flag, err)) {
+                            if (b == 0 || two)
+                                asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                                             :: "l"(reinterpret_cast<uint64_t>(&P.tf)), "r"(rx0 + PX * b), "r"(ry0), "r"(z),
+                                                "r"(smem_u32(sF) + b * OUT_F)
+                                             : "memory");
+                            if (b == 1)
+                                asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                                             :: "l"(reinterpret_cast<uint64_t>(&P.tc)), "r"(rx0), "r"(ry0), "r"(z), "r"(smem_u32(sC))
+                                             : "memory");
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                        }
+                        mbar_arrive(bar_vfree + 8 * b);
+                    }
+                    mbar_arrive(bar_cfree);
                 }
             }
         } else {
-            // epilogue: warp w drains TMEM lane quadrant w % 4, pooled columns of part (w - 2) / 4
+            // epilogue: two groups of 8 warps, each on the tiles of one accumulator (one
+            // N-tile of the pair), so that one group's waits (for the MMA, its tensor-memory
+            // loads) are filled by the other's arithmetic; warp w drains TMEM lane quadrant
+            // w % 4
             const int quad = warp & 3;
-            const EpiArgs ea{tmem + ((uint32_t)(quad * 32) << 16), quad * 32 + lane, (warp - 2) >> 2, cx0, cy0, W2, H2,
-                             lam, cx0 >= 0 && cy0 >= 0 && cx0 + CX <= W2 && cy0 + CY <= H2};
+            const uint32_t b = warp >= 2 + EPI_WARPS / 2 ? 1u : 0u;
+            const int tcx0 = cx0 + 2 * PX * (int)b;
+            const EpiArgs ea{tmem + ((uint32_t)(quad * 32) << 16) + b * 256, quad * 32 + lane, ((warp - 2) >> 2) & 1, (int)b, tcx0,
+                             cy0, W2, H2, lam, tcx0 >= 0 && cy0 >= 0 && tcx0 + CX <= W2 && cy0 + CY <= H2};
             // FP8: 1/16 times the inverse operand scales (powers of two, exact), the
             // patch's scale loaded before the accumulator wait so its latency hides there
             const float mult_b = FMT == FMT_E4M3 ? 0.0625f * (1.0f / s_b) : 0.0625f;
             for (int j = 0; j < nt; j++) {
-                const uint32_t ai = acc_it + j, b = ai & 1, aph = (ai >> 1) & 1;
-                float mult = mult_b;
-                if (FMT == FMT_E4M3) {
-                    const int p = (m0 + j) * BM + ea.row;
-                    mult = mult_b * __ldg(inv_sa + p);       // inv_sa covers every row of every M-tile
+                const uint32_t it = a_it + j, aph = (b ? acc1_it + j : it) & 1;
+                auto values_free = [&] { mbar_wait(bar_vfree + 8 * b, (it & 1) ^ 1, abort_flag, err); };
+                auto codes_free = [&] { mbar_wait(bar_cfree, (it & 1) ^ 1, abort_flag, err); };
+                if (b && !two) {
+                    codes_free();                            // nothing to drain: one arrival per tile
+                } else {
+                    float mult = mult_b;
+                    if (FMT == FMT_E4M3) {
+                        const int p = (m0 + j) * BM + ea.row;
+                        mult = mult_b * __ldg(inv_sa + p);   // inv_sa covers every row of every M-tile
+                    }
+                    // after a failed (bounded) wait the tile is skipped, the arrivals go on
+                    if (mbar_wait(bar_acc_full + 8 * b, aph, abort_flag, err)) {
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        epilogue_tile(ea, bar_acc_empty + 8 * b, mult, sF + b * (OUT_F / 4), sC, values_free, codes_free);
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    }
                 }
-                // a failed (bounded) wait has set the abort flag: this thread skips the
-                // tile but still meets the barrier, after which every thread sees the flag
-                if (mbar_wait(bar_acc_full + 8 * b, aph, abort_flag, err)) {
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    epilogue_tile(ea, b, bar_acc_empty + 8 * b, mult, sF + b * (OUT_F / 4), sC + b * OUT_C);
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                }
-                // one barrier per tile: before it the leader also waits until the store
-                // of the previous tile has read its staging buffer, which the next tile
-                // fills (the staging is double-buffered)
-                if (store_leader) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                epi_barrier();
-                if (*abort_flag) break;
-                float* stf = sF + b * (OUT_F / 4);
-                unsigned char* stc = sC + b * OUT_C;
-                if (store_leader) {
-                    const int z = (m0 + j) * BM;
-                    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                                 :: "l"(reinterpret_cast<uint64_t>(&P.tf)), "r"(rx0), "r"(ry0), "r"(z), "r"(smem_u32(stf))
-                                 : "memory");
-                    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                                 :: "l"(reinterpret_cast<uint64_t>(&P.tc)), "r"(rx0), "r"(ry0), "r"(z), "r"(smem_u32(stc))
-                                 : "memory");
-                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_staged + 8 * b);
             }
         }
         a_it += nt;
-        acc_it += nt;
+        if (two) acc1_it += nt;
         __syncthreads();   // the epilogue has consumed every accumulator: the tensor core is done with sB
         if (*abort_flag) break;
     }
-    if (store_leader) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (warp == STORE_WARP && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     __syncthreads();
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(512));
 }
 
 // 3-D map of a pooled level-0 array [n0][mh][pitch] (elements of `esize` bytes),
-// logical extent mw x mh x n0, box 16 x 3 x 128, staged with the given swizzle.
-bool make_map(CUtensorMap* m, void* base, CUtensorMapDataType dt, int esize, const DmGeom& g, int n0, CUtensorMapSwizzle sw) {
+// logical extent mw x mh x n0, box cols x 3 x 128, staged with the given swizzle.
+bool make_map(CUtensorMap* m, void* base, CUtensorMapDataType dt, int esize, const DmGeom& g, int n0, int cols,
+              CUtensorMapSwizzle sw) {
     const cuuint64_t dims[3] = {(cuuint64_t)g.dw[1], (cuuint64_t)g.dh[1], (cuuint64_t)n0};
     const cuuint64_t strides[2] = {(cuuint64_t)g.pitch(1) * esize, (cuuint64_t)g.pitch(1) * g.dh[1] * esize};
-    const cuuint32_t box[3] = {PX, PY, BM};
+    const cuuint32_t box[3] = {(cuuint32_t)cols, PY, BM};
     return dm_encode_tiled(m, dt, 3, base, dims, strides, box, sw);
+}
+
+int tc_sm_count() {
+    int dev = 0, nsm = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return nsm;
 }
 
 template <int FMT>
 cudaError_t launch_tc(const L0Batch& B, float lam, cudaStream_t st) {
     using F = Fmt<FMT>;
-    int dev = 0, nsm = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int nsm = tc_sm_count();
     static std::atomic<unsigned long long> smem_done{0};
     cudaError_t ea = dm_smem_opt_in(reinterpret_cast<const void*>(k_corr0_tc<FMT>), (int)F::SMEM, smem_done);
     if (ea != cudaSuccess) return ea;
@@ -628,10 +729,24 @@ cudaError_t prepare_pair(const DmGeom& g, int precision, const float* d1, const 
     memset(q, 0, sizeof(*q));
     const int n0 = n_rows < 0 ? g.npatch(0) : n_rows;
     const int n_mtiles = (n0 + BM - 1) / BM;
+    // work units: pairs of N-tiles times chunks of at most m_chunk M-tiles.  The chunks
+    // are made smaller where that fills the last round of the SMs better: rounds times
+    // (tiles + about one tile's time for the unit's operand), by 2 % or more (256x256
+    // BF16: one chunk of 32 tiles 263 us, this choice 209; the choice does not depend on
+    // whether half a tile or three stand for the operand).
+    const int pairs = ((g.dw[1] + SX - 1) / SX) * ((g.dh[1] + PY - 1) / PY), nsm = tc_sm_count();
     if (m_chunk < 1) m_chunk = 1;
-    // values: 64-byte box rows staged with the 64-byte swizzle (see pool_out)
-    if (!make_map(&q->tf, pooled0, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g, n0, CU_TENSOR_MAP_SWIZZLE_64B) ||
-        !make_map(&q->tc, amax0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g, n0, CU_TENSOR_MAP_SWIZZLE_NONE))
+    int best = 0;
+    double best_cost = 0.0;
+    for (int k = (n_mtiles + m_chunk - 1) / m_chunk; k <= n_mtiles && k < 64; k++) {
+        const int c = (n_mtiles + k - 1) / k;
+        const double cost = (double)(((long long)pairs * ((n_mtiles + c - 1) / c) + nsm - 1) / nsm) * (c + 1);
+        if (best == 0 || cost < 0.98 * best_cost) { best = c; best_cost = cost; }
+    }
+    if (best > 0) m_chunk = best;
+    // box rows of 64 and 32 bytes staged with the swizzle of that span (see pool_out, stage_codes)
+    if (!make_map(&q->tf, pooled0, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g, n0, PX, CU_TENSOR_MAP_SWIZZLE_64B) ||
+        !make_map(&q->tc, amax0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g, n0, SX, CU_TENSOR_MAP_SWIZZLE_32B))
         return cudaErrorNotSupported;
     unsigned char* apack = reinterpret_cast<unsigned char*>(abuf);
     q->g = g;
@@ -640,7 +755,7 @@ cudaError_t prepare_pair(const DmGeom& g, int precision, const float* d1, const 
     q->err = reinterpret_cast<int*>(status);
     q->n_mtiles = n_mtiles;
     q->m_chunk = m_chunk;
-    q->units = ((g.dw[1] + PX - 1) / PX) * ((g.dh[1] + PY - 1) / PY) * ((n_mtiles + m_chunk - 1) / m_chunk);
+    q->units = pairs * ((n_mtiles + m_chunk - 1) / m_chunk);
     cudaError_t e;
     if (precision == DM_FP8_E4M3) {
         const size_t a_bytes = dm_align((size_t)n_mtiles * Fmt<FMT_E4M3>::A_TILE);
