@@ -13,11 +13,12 @@
 // match lands on a coarse level, SOR ordering) are stated at each kernel.
 //
 // The SOR sweeps are sequential in time (each half-sweep needs the other
-// colour's previous values), so the launch count, not the arithmetic, bounds
-// the solver: the smallest levels (up to 1024 pixels) run entirely in one
-// CTA with their state in shared memory; larger levels run 8 half-sweeps per launch, temporally blocked in
-// shared memory (a tile plus an 8-pixel halo), which gives the same bits as
-// 8 global half-sweeps.
+// colour's previous values), so the latency of a half-sweep and the launches,
+// not the arithmetic, bound the solver: the smaller levels (up to 4096 pixels) run
+// entirely in one CTA; larger levels run 8 half-sweeps per launch, temporally blocked
+// (a tile plus an 8-pixel halo), which gives the same bits as 8 global half-sweeps.
+// In both a thread keeps the weights and increments of its pixels in registers and
+// reads only its neighbours' current values from shared memory.
 #include <math.h>
 
 #include "dm_internal.cuh"
@@ -233,19 +234,18 @@ struct DfPix {
     float ps, a11, a12, a22, b1, b2;
 };
 
-__device__ __forceinline__ DfPix df_weights_vals(float u, float du, float v, float dv, bool has_r, float ur, float dur,
-                                                 float vr, float dvr, bool has_d, float ud, float dud, float vd, float dvd,
-                                                 const float* d, float alpha, float mc, float mu, float mv,
+__device__ __forceinline__ DfPix df_weights_vals(float u, float du, float v, float dv, bool has_r, float Ur, float Vr,
+                                                 bool has_d, float Ud, float Vd, const float* d, float alpha, float mc, float mu, float mv,
                                                  const DfConst& k) {
     const float U = __fadd_rn(u, du), V = __fadd_rn(v, dv);
     float ux = 0.0f, uy = 0.0f, vx = 0.0f, vy = 0.0f;
     if (has_r) {
-        ux = __fsub_rn(__fadd_rn(ur, dur), U);
-        vx = __fsub_rn(__fadd_rn(vr, dvr), V);
+        ux = __fsub_rn(Ur, U);
+        vx = __fsub_rn(Vr, V);
     }
     if (has_d) {
-        uy = __fsub_rn(__fadd_rn(ud, dud), U);
-        vy = __fsub_rn(__fadd_rn(vd, dvd), V);
+        uy = __fsub_rn(Ud, U);
+        vy = __fsub_rn(Vd, V);
     }
     DfPix r;
     const float s2 = __fadd_rn(__fadd_rn(__fadd_rn(__fmul_rn(ux, ux), __fmul_rn(uy, uy)), __fmul_rn(vx, vx)), __fmul_rn(vy, vy));
@@ -288,8 +288,9 @@ __device__ __forceinline__ void df_weights_at(const DfLevel& L, const DfConst& k
     const long long r = hr ? o + 1 : o, dn = hd ? o + L.w : o;
     float d[11];
     df_load_d(L.D, L.n, o, d);
-    const DfPix q = df_weights_vals(L.u[o], L.du[o], L.v[o], L.dv[o], hr, L.u[r], L.du[r], L.v[r], L.dv[r], hd, L.u[dn],
-                                    L.du[dn], L.v[dn], L.dv[dn], d, L.alpha[o], L.mc[o], L.mu[o], L.mv[o], k);
+    const DfPix q = df_weights_vals(L.u[o], L.du[o], L.v[o], L.dv[o], hr, __fadd_rn(L.u[r], L.du[r]),
+                                    __fadd_rn(L.v[r], L.dv[r]), hd, __fadd_rn(L.u[dn], L.du[dn]),
+                                    __fadd_rn(L.v[dn], L.dv[dn]), d, L.alpha[o], L.mc[o], L.mu[o], L.mv[o], k);
     const long long n = L.n;
     L.ps[o] = q.ps;
     L.A[o] = q.a11;
@@ -299,27 +300,87 @@ __device__ __forceinline__ void df_weights_at(const DfLevel& L, const DfConst& k
     L.A[4 * n + o] = q.b2;
 }
 
-// One SOR relaxation of a pixel from its existing 4-neighbours (left, right,
-// up, down, compacted into nb[0..nn)): edge weight (ps_o + ps_p) / 2,
-//   du = (1 - omega) du + omega (b1 + sum w (du_p + u_p - u_o) - A12 dv) / (A11 + sum w),
-// then dv the same way with the new du.  Get(p, ps, du, u, dv, v) reads a neighbour.
-template <class Get>
-__device__ __forceinline__ void df_sor_vals(int nn, const int* nb, Get get, float pso, float uo, float vo, float a11,
-                                            float a12, float a22, float b1, float b2, const DfConst& k, float& du,
-                                            float& dv) {
-    float sw = 0.0f, su = 0.0f, sv = 0.0f;
-    for (int j = 0; j < nn; j++) {
-        float psp, dup, up, dvp, vp;
-        get(nb[j], psp, dup, up, dvp, vp);
-        const float we = __fmul_rn(0.5f, __fadd_rn(pso, psp));
-        sw = __fadd_rn(sw, we);
-        su = __fadd_rn(su, __fmul_rn(we, __fsub_rn(__fadd_rn(dup, up), uo)));
-        sv = __fadd_rn(sv, __fmul_rn(we, __fsub_rn(__fadd_rn(dvp, vp), vo)));
-    }
-    const float nu = __fsub_rn(__fadd_rn(b1, su), __fmul_rn(a12, dv));
-    du = __fadd_rn(__fmul_rn(k.one_m_omega, du), __fmul_rn(k.omega, __fdiv_rn(nu, __fadd_rn(a11, sw))));
-    const float nv = __fsub_rn(__fadd_rn(b2, sv), __fmul_rn(a12, du));
-    dv = __fadd_rn(__fmul_rn(k.one_m_omega, dv), __fmul_rn(k.omega, __fdiv_rn(nv, __fadd_rn(a22, sw))));
+// ---------------------------------------------------------------------------
+// Red-black SOR in a CTA.  One relaxation of a pixel o from its existing
+// 4-neighbours p (left, right, up, down), edge weights w_p = (ps_o + ps_p) / 2:
+//   du = (1 - omega) du + omega (b1 + sum w_p ((du_p + u_p) - u_o) - A12 dv) / (A11 + sum w_p),
+// then dv the same way with the new du.
+//
+// A thread owns pairs of horizontally neighbouring pixels, one of each colour, so
+// every thread updates a pixel in every half-sweep.  What does not change during
+// the sweeps is formed once: the edge weights (0 for a missing neighbour: the
+// terms it adds are zeros, which leave the sums unchanged), the two diagonals and
+// their reciprocals.  Shared memory holds, in one plane per colour (a warp's
+// accesses are then consecutive), the sums (du + u, dv + v) that the neighbours
+// read -- one 8-byte load each -- and the constants of the pixel's own update.
+// Against reading ps, du, u, dv, v of every neighbour
+// and two divisions per update this shortens the chain of an update to less than half:
+// the blocked launch of a level of a few tiles 12.6 -> 7.4 us, of 1024x436 45.7 -> 29.1,
+// a one-CTA level 220 -> 100 us; with the launches of a fixed-point step overlapped
+// (programmatic dependence) a 1024x436 pair 39.2 -> 26.3 -> 20.3 ms.
+constexpr int SOR_INV = 7;       // planes of constants: A12, b1, b2, A11 + w, 1 / that, A22 + w, 1 / that
+
+struct SorPx {
+    float wl, wr, wu, wd;        // edge weights
+    float u, v, du, dv;
+};
+
+// a / d correctly rounded, y = RN(1 / d): the quotient estimate with two remainder
+// corrections (Markstein: the remainder of an fma is exact, and with a correctly
+// rounded reciprocal the correction of a quotient that is off by less than an ulp
+// rounds correctly).  Outside the range where no remainder can underflow -- and
+// for the d that dm_sor_setup marks with lo = infinity -- the division itself.
+__device__ __forceinline__ float df_div(float a, float d, float y, float lo) {
+    const float m = fabsf(a);
+    if (!(m >= lo && m <= 1.0e24f)) return __fdiv_rn(a, d);
+    float q = __fmul_rn(a, y);
+    q = __fmaf_rn(__fmaf_rn(-d, q, a), y, q);
+    return __fmaf_rn(__fmaf_rn(-d, q, a), y, q);
+}
+
+// The constants of one pixel from its system and its neighbours' ps (has_*: the
+// neighbour exists); returns false where a diagonal lies outside df_div's range.
+__device__ __forceinline__ bool sor_setup(SorPx& p, float* inv, int stride, float pso, bool hl, float psl, bool hr, float psr,
+                                          bool hu, float psu, bool hd, float psd, float a11, float a12, float a22, float b1,
+                                          float b2) {
+    p.wl = hl ? __fmul_rn(0.5f, __fadd_rn(pso, psl)) : 0.0f;
+    p.wr = hr ? __fmul_rn(0.5f, __fadd_rn(pso, psr)) : 0.0f;
+    p.wu = hu ? __fmul_rn(0.5f, __fadd_rn(pso, psu)) : 0.0f;
+    p.wd = hd ? __fmul_rn(0.5f, __fadd_rn(pso, psd)) : 0.0f;
+    const float sw = __fadd_rn(__fadd_rn(__fadd_rn(p.wl, p.wr), p.wu), p.wd);
+    const float d1 = __fadd_rn(a11, sw), d2 = __fadd_rn(a22, sw);
+    inv[0] = a12;
+    inv[stride] = b1;
+    inv[2 * stride] = b2;
+    inv[3 * stride] = d1;
+    inv[4 * stride] = __frcp_rn(d1);
+    inv[5 * stride] = d2;
+    inv[6 * stride] = __frcp_rn(d2);
+    return fminf(d1, d2) >= 1.0e-12f && fmaxf(d1, d2) <= 1.0e12f;
+}
+
+// The other colour's neighbours of a pixel of pair e (planes of `pw` pairs per row): the
+// pixel of colour c lies at column 2 i + off of its row, its left and right
+// neighbours in pairs e - 1 + off and e + off, the upper and lower ones in e -+ pw.
+// (A neighbour that does not exist has weight 0, so any finite value serves: the
+// planes have `pw` guard elements before and after.)
+__device__ __forceinline__ void sor_update(SorPx& p, float2* mine, const float2* other, int off, int pw, const float* inv,
+                                           int stride, float lo, const DfConst& k) {
+    const float2 l = other[off - 1], r = other[off], t = other[-pw], b = other[pw];
+    const float a12 = inv[0], b1 = inv[stride], b2 = inv[2 * stride];
+    const float d1 = inv[3 * stride], y1 = inv[4 * stride], d2 = inv[5 * stride], y2 = inv[6 * stride];
+    float su = __fmul_rn(p.wl, __fsub_rn(l.x, p.u)), sv = __fmul_rn(p.wl, __fsub_rn(l.y, p.v));
+    su = __fadd_rn(su, __fmul_rn(p.wr, __fsub_rn(r.x, p.u)));
+    sv = __fadd_rn(sv, __fmul_rn(p.wr, __fsub_rn(r.y, p.v)));
+    su = __fadd_rn(su, __fmul_rn(p.wu, __fsub_rn(t.x, p.u)));
+    sv = __fadd_rn(sv, __fmul_rn(p.wu, __fsub_rn(t.y, p.v)));
+    su = __fadd_rn(su, __fmul_rn(p.wd, __fsub_rn(b.x, p.u)));
+    sv = __fadd_rn(sv, __fmul_rn(p.wd, __fsub_rn(b.y, p.v)));
+    const float nu = __fsub_rn(__fadd_rn(b1, su), __fmul_rn(a12, p.dv));
+    p.du = __fadd_rn(__fmul_rn(k.one_m_omega, p.du), __fmul_rn(k.omega, df_div(nu, d1, y1, lo)));
+    const float nv = __fsub_rn(__fadd_rn(b2, sv), __fmul_rn(a12, p.du));
+    p.dv = __fadd_rn(__fmul_rn(k.one_m_omega, p.dv), __fmul_rn(k.omega, df_div(nv, d2, y2, lo)));
+    *mine = make_float2(__fadd_rn(p.du, p.u), __fadd_rn(p.dv, p.v));
 }
 
 __global__ void k_df_weights(DfLevel L, DfConst k) {
@@ -328,8 +389,8 @@ __global__ void k_df_weights(DfLevel L, DfConst k) {
 }
 
 // Temporally blocked red-black SOR: a CTA owns a TB_W x TB_H tile and stages
-// it with a halo of S pixels (S = the half-sweeps of this launch, <= TB_S) in
-// shared memory, then runs S half-sweeps there, colour start, start + 1, ...
+// it with a halo of S pixels (S = the half-sweeps of this launch, even, <= TB_S) in
+// shared memory and registers, then runs S half-sweeps there, colours 0, 1, 0, ...
 // Half-sweep j updates the pixels of its colour in the staged region shrunk by
 // j + 1 on every side that is not the image border: their neighbours then
 // hold exactly the values the global sweep would give them, so after S
@@ -339,74 +400,104 @@ __global__ void k_df_weights(DfLevel L, DfConst k) {
 // L.du / L.dv and written to a second pair of buffers (ping-pong between
 // launches): no CTA ever sees another's updates of the same launch.
 constexpr int TB_W = 32, TB_H = 16, TB_S = 8;
-constexpr int TB_LW = TB_W + 2 * TB_S, TB_LH = TB_H + 2 * TB_S, TB_LN = TB_LW * TB_LH;
-constexpr size_t TB_SMEM = (size_t)TB_LN * 10 * sizeof(float);
+constexpr int TB_LW = TB_W + 2 * TB_S, TB_LH = TB_H + 2 * TB_S;
+constexpr int TB_PW = TB_LW / 2, TB_PAIRS = TB_PW * TB_LH;       // 24 x 32 pairs, one per thread
+constexpr int TB_THREADS = TB_PAIRS;
+constexpr int TB_PLANE = TB_PAIRS + 2 * TB_PW;                   // with guards
+constexpr size_t TB_SMEM = (size_t)(4 * TB_PLANE + 2 * SOR_INV * TB_PAIRS) * sizeof(float);
+static_assert(TB_S % 2 == 0 && TB_W % 2 == 0, "a launch starts with colour 0 and the staged region at an even column");
 
-constexpr int TB_THREADS = 1024;                  // a tile's half-sweep is short: many threads, short latency
-
-__global__ void __launch_bounds__(TB_THREADS) k_df_sor_tb(DfLevel L, DfConst k, int start_color, int S, float* __restrict__ out_du,
-                                                   float* __restrict__ out_dv) {
+// Launches of one fixed-point step follow one another with programmatic dependence:
+// what a launch reads that the one before it does not write (u, v, ps, A) is staged
+// before it waits for that one (`early`; the first launch waits first, since the
+// kernel before it writes them), and only its increments after.  Every launch lets
+// its successor start after its own wait, so a launch that starts early knows the
+// kernel before its predecessor to have ended.
+__global__ void __launch_bounds__(TB_THREADS, 2) k_df_sor_tb(DfLevel L, DfConst k, int S, int early, float* __restrict__ out_du,
+                                                             float* __restrict__ out_dv) {
+    if (!early) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
     extern __shared__ __align__(16) float sm[];
-    float* sdu = sm;
-    float* sdv = sm + TB_LN;
-    float* su_ = sm + 2 * TB_LN;
-    float* sv_ = sm + 3 * TB_LN;
-    float* sps = sm + 4 * TB_LN;
-    float* sA = sm + 5 * TB_LN;          // [5][TB_LN]
+    // per colour: the sums, the constants of this thread's pixel
+    float2* cur[2] = {reinterpret_cast<float2*>(sm) + TB_PW + threadIdx.x,
+                      reinterpret_cast<float2*>(sm) + TB_PLANE + TB_PW + threadIdx.x};
+    float* inv[2] = {sm + 4 * TB_PLANE + threadIdx.x, sm + 4 * TB_PLANE + SOR_INV * TB_PAIRS + threadIdx.x};
+    float* sps = sm;                                     // [TB_LH][TB_LW], before the sums take its place
     const int tiles_x = (L.w + TB_W - 1) / TB_W;
     const int tx0 = (blockIdx.x % tiles_x) * TB_W, ty0 = (blockIdx.x / tiles_x) * TB_H;
     const int tx1 = min(tx0 + TB_W, L.w), ty1 = min(ty0 + TB_H, L.h);
-    const int lx0 = max(tx0 - S, 0), ly0 = max(ty0 - S, 0);
+    const int lx0 = max(tx0 - S, 0) & ~1, ly0 = max(ty0 - S, 0);
     const int lx1 = min(tx1 + S, L.w), ly1 = min(ty1 + S, L.h);
-    const int lw = lx1 - lx0, lh = ly1 - ly0, ln = lw * lh;
+    const int lw = lx1 - lx0, lh = ly1 - ly0;
     const long long n = L.n;
-    for (int i = threadIdx.x; i < ln; i += blockDim.x) {
-        const long long o = (long long)(ly0 + i / lw) * L.w + (lx0 + i % lw);
-        sdu[i] = L.du[o];
-        sdv[i] = L.dv[o];
-        su_[i] = L.u[o];
-        sv_[i] = L.v[o];
-        sps[i] = L.ps[o];
+    const int i = threadIdx.x % TB_PW, y = threadIdx.x / TB_PW, gy = ly0 + y;
+    const int flip = (lx0 + gy) & 1;                     // offset of colour 0 in this row's pairs
+    // colour c of the pair lies at column 2 i + (c ^ flip)
+    SorPx px[2];
+    int act[2];                                          // half-sweeps in which the pixel is updated: j < act
+    float ps[2], A[2][5];
+    bool in[2];
 #pragma unroll
-        for (int j = 0; j < 5; j++) sA[j * TB_LN + i] = L.A[j * n + o];
+    for (int c = 0; c < 2; c++) {
+        const int x = 2 * i + (c ^ flip);
+        in[c] = x < lw && y < lh;
+        const long long o = in[c] ? (long long)gy * L.w + (lx0 + x) : 0;
+        px[c].u = L.u[o];
+        px[c].v = L.v[o];
+        ps[c] = L.ps[o];
+#pragma unroll
+        for (int j = 0; j < 5; j++) A[c][j] = L.A[j * n + o];
+        sps[y * TB_LW + x] = ps[c];
     }
     __syncthreads();
-    auto get = [&](int p, float& ps, float& du, float& u, float& dv, float& v) {
-        ps = sps[p]; du = sdu[p]; u = su_[p]; dv = sdv[p]; v = sv_[p];
-    };
-    for (int j = 0; j < S; j++) {
-        const int color = (start_color + j) & 1;
-        const int ax0 = lx0 > 0 ? lx0 + j + 1 : lx0, ay0 = ly0 > 0 ? ly0 + j + 1 : ly0;
-        const int ax1 = lx1 < L.w ? lx1 - j - 1 : lx1, ay1 = ly1 < L.h ? ly1 - j - 1 : ly1;
-        const int aw = ax1 - ax0, ah = ay1 - ay0;
-        if (aw > 0 && ah > 0) {
-            const int half = (aw + 1) / 2;
-            for (int i = threadIdx.x; i < half * ah; i += blockDim.x) {
-                const int gy = ay0 + i / half;
-                const int gx = ax0 + 2 * (i % half) + ((gy + ax0 + color) & 1);
-                if (gx >= ax1) continue;
-                const int p = (gy - ly0) * lw + (gx - lx0);
-                int nb[4], nn = 0;
-                if (gx > 0) nb[nn++] = p - 1;
-                if (gx + 1 < L.w) nb[nn++] = p + 1;
-                if (gy > 0) nb[nn++] = p - lw;
-                if (gy + 1 < L.h) nb[nn++] = p + lw;
-                float du = sdu[p], dv = sdv[p];
-                df_sor_vals(nn, nb, get, sps[p], su_[p], sv_[p], sA[p], sA[TB_LN + p], sA[2 * TB_LN + p],
-                            sA[3 * TB_LN + p], sA[4 * TB_LN + p], k, du, dv);
-                sdu[p] = du;
-                sdv[p] = dv;
-            }
-        }
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        const int x = 2 * i + (c ^ flip), gx = lx0 + x;
+        const bool hl = gx > 0, hr = gx + 1 < L.w, hu = gy > 0, hd = gy + 1 < L.h;
+        auto at = [&](int yy, int xx) { return xx >= 0 && xx < TB_LW && yy >= 0 && yy < TB_LH ? sps[yy * TB_LW + xx] : 0.0f; };
+        // half-sweep j updates the staged region shrunk by j + 1 on sides that are not
+        // the image border
+        act[c] = in[c] ? S : 0;
+        if (lx0 > 0) act[c] = min(act[c], x);
+        if (ly0 > 0) act[c] = min(act[c], y);
+        if (lx1 < L.w) act[c] = min(act[c], lw - 1 - x);
+        if (ly1 < L.h) act[c] = min(act[c], lh - 1 - y);
+        const bool good = sor_setup(px[c], inv[c], TB_PAIRS, ps[c], hl, at(y, x - 1), hr, at(y, x + 1), hu, at(y - 1, x),
+                                    hd, at(y + 1, x), A[c][0], A[c][1], A[c][2], A[c][3], A[c][4]);
+        ok = ok && (good || act[c] <= 0);
+    }
+    __syncthreads();                                     // ps read
+    if (early) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        const long long o = in[c] ? (long long)gy * L.w + (lx0 + 2 * i + (c ^ flip)) : 0;
+        px[c].du = __ldcg(L.du + o);                     // (written by the launch before)
+        px[c].dv = __ldcg(L.dv + o);
+        cur[c][0] = make_float2(__fadd_rn(px[c].du, px[c].u), __fadd_rn(px[c].dv, px[c].v));
+        if (threadIdx.x < TB_PW) cur[c][-TB_PW] = cur[c][TB_PAIRS] = make_float2(0.0f, 0.0f);
+    }
+    const float lo = ok ? 1.0e-24f : INFINITY;
+    __syncthreads();
+    for (int j = 0; j < S; j += 2) {
+        if (j < act[0]) sor_update(px[0], cur[0], cur[1], flip, TB_PW, inv[0], TB_PAIRS, lo, k);
+        __syncthreads();
+        if (j + 1 < act[1]) sor_update(px[1], cur[1], cur[0], flip ^ 1, TB_PW, inv[1], TB_PAIRS, lo, k);
         __syncthreads();
     }
-    const int ow = tx1 - tx0;
-    for (int i = threadIdx.x; i < ow * (ty1 - ty0); i += blockDim.x) {
-        const int gx = tx0 + i % ow, gy = ty0 + i / ow;
-        const int p = (gy - ly0) * lw + (gx - lx0);
-        const long long o = (long long)gy * L.w + gx;
-        out_du[o] = sdu[p];
-        out_dv[o] = sdv[p];
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        const int gx = lx0 + 2 * i + (c ^ flip);
+        if (gx >= tx0 && gx < tx1 && gy >= ty0 && gy < ty1) {
+            const long long o = (long long)gy * L.w + gx;
+            out_du[o] = px[c].du;
+            out_dv[o] = px[c].dv;
+        }
     }
 }
 
@@ -418,83 +509,86 @@ __global__ void k_df_update(float* __restrict__ u, float* __restrict__ v, const 
     }
 }
 
-// A whole small level in one CTA with its state in shared memory: u, v, du,
-// dv, ps and the system (10 floats per pixel); n_fixed x (weights, then
-// n_sor red-black sweeps) with block barriers between the passes, then
-// w += dw.  The same per-pixel arithmetic as the multi-launch path.
+// A whole small level in one CTA: n_fixed x (weights, then n_sor red-black sweeps)
+// with block barriers between the passes, then w += dw.  The same per-pixel
+// arithmetic as the multi-launch path.  One pair of pixels per thread.
 constexpr int DF_SMALL_THREADS = 1024;
-// Pixels of a level solved by one CTA: above about a thousand pixels a single
-// SM is slower than the blocked launches (1024x436 pair: 43.0 ms with 5120
-// and 256-thread blocked CTAs, 39.4 ms with 1024 and 1024 threads).  At most
-// 5120 (200 KB of shared memory).
-constexpr int DF_SMALL_MAX = 1024;
-constexpr size_t DF_SMALL_SMEM = (size_t)DF_SMALL_MAX * 10 * sizeof(float);
-static_assert(DF_SMALL_MAX <= 5120, "small-level state must fit shared memory");
+// Pairs of a level solved by one CTA (a row of w pixels holds (w + 1) / 2): with two
+// pairs per thread, up to 2048, a 1024x436 pair took 0.4 ms longer (spilled registers).
+constexpr int DF_SMALL_PAIRS = DF_SMALL_THREADS;
+constexpr size_t DF_SMALL_SMEM = (size_t)(DF_SMALL_PAIRS * 2 * (2 + SOR_INV + 1) + 8 * DF_SMALL_PAIRS) * sizeof(float);   // sums, constants, psi_s, guards
 
 __global__ void __launch_bounds__(DF_SMALL_THREADS) k_df_level_small(DfLevel L, DfConst k, int n_fixed, int n_sor) {
     extern __shared__ __align__(16) float sm[];
-    const int n = (int)L.n, w = L.w, h = L.h;
-    float* su_ = sm;
-    float* sv_ = sm + n;
-    float* sdu = sm + 2 * n;
-    float* sdv = sm + 3 * n;
-    float* sps = sm + 4 * n;
-    float* sA = sm + 5 * n;              // [5][n]
-    for (int o = threadIdx.x; o < n; o += blockDim.x) {
-        su_[o] = L.u[o];
-        sv_[o] = L.v[o];
-        sdu[o] = 0.0f;
-        sdv[o] = 0.0f;
+    const int w = L.w, h = L.h, pw = (w + 1) / 2, np = pw * h, plane = np + 2 * pw;
+    const long long n = L.n;
+    float2* cur[2] = {reinterpret_cast<float2*>(sm) + pw, reinterpret_cast<float2*>(sm) + plane + pw};
+    float* inv[2] = {sm + 4 * plane, sm + 4 * plane + SOR_INV * np};
+    float* sps[2] = {sm + 4 * plane + 2 * SOR_INV * np, sm + 4 * plane + (2 * SOR_INV + 1) * np};      // psi_s per colour
+    const int e = threadIdx.x, y = e / pw, i = e - y * pw, flip = y & 1;
+    SorPx px[2];                                         // per colour, at column 2 i + (c ^ flip)
+    bool in[2];
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        SorPx& p = px[c];
+        const int x = 2 * i + (c ^ flip);
+        in[c] = e < np && x < w;
+        p.u = p.v = p.du = p.dv = p.wl = p.wr = p.wu = p.wd = 0.0f;
+        if (in[c]) {
+            p.u = L.u[(long long)y * w + x];
+            p.v = L.v[(long long)y * w + x];
+        }
+        if (e < np) cur[c][e] = make_float2(p.u, p.v);   // du = dv = 0
+        if (e < pw) cur[c][e - pw] = cur[c][np + e] = make_float2(0.0f, 0.0f);
     }
     __syncthreads();
-    auto get = [&](int p, float& ps, float& du, float& u, float& dv, float& v) {
-        ps = sps[p]; du = sdu[p]; u = su_[p]; dv = sdv[p]; v = sv_[p];
-    };
-    const int half = (w + 1) / 2;
     for (int it = 0; it < n_fixed; it++) {
-        for (int o = threadIdx.x; o < n; o += blockDim.x) {
-            const int x = o % w, y = o / w;
-            const bool hr = x + 1 < w, hd = y + 1 < h;
-            const int r = hr ? o + 1 : o, dn = hd ? o + w : o;
+        // systems and smoothness weights: u + du and v + dv of the right and lower
+        // neighbours are the sums in `cur`
+        DfPix a[2];
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            if (!in[c]) continue;
+            const SorPx& p = px[c];
+            const int x = 2 * i + (c ^ flip);
+            const long long o = (long long)y * w + x;
+            const float2 r = cur[c ^ 1][e + (c ^ flip)], b = cur[c ^ 1][e + pw];
             float d[11];
-            df_load_d(L.D, L.n, o, d);
-            const DfPix q = df_weights_vals(su_[o], sdu[o], sv_[o], sdv[o], hr, su_[r], sdu[r], sv_[r], sdv[r], hd, su_[dn],
-                                            sdu[dn], sv_[dn], sdv[dn], d, L.alpha[o], L.mc[o], L.mu[o], L.mv[o], k);
-            sps[o] = q.ps;
-            sA[o] = q.a11;
-            sA[n + o] = q.a12;
-            sA[2 * n + o] = q.a22;
-            sA[3 * n + o] = q.b1;
-            sA[4 * n + o] = q.b2;
+            df_load_d(L.D, n, o, d);
+            a[c] = df_weights_vals(p.u, p.du, p.v, p.dv, x + 1 < w, r.x, r.y, y + 1 < h, b.x, b.y, d, L.alpha[o], L.mc[o],
+                                   L.mu[o], L.mv[o], k);
+            sps[c][e] = a[c].ps;
         }
         __syncthreads();
-        for (int s = 0; s < n_sor; s++)
-            for (int color = 0; color < 2; color++) {
-                for (int i = threadIdx.x; i < half * h; i += blockDim.x) {
-                    const int y = i / half;
-                    const int x = 2 * (i % half) + ((y + color) & 1);
-                    if (x >= w) continue;
-                    const int p = y * w + x;
-                    int nb[4], nn = 0;
-                    if (x > 0) nb[nn++] = p - 1;
-                    if (x + 1 < w) nb[nn++] = p + 1;
-                    if (y > 0) nb[nn++] = p - w;
-                    if (y + 1 < h) nb[nn++] = p + w;
-                    float du = sdu[p], dv = sdv[p];
-                    df_sor_vals(nn, nb, get, sps[p], su_[p], sv_[p], sA[p], sA[n + p], sA[2 * n + p], sA[3 * n + p],
-                                sA[4 * n + p], k, du, dv);
-                    sdu[p] = du;
-                    sdv[p] = dv;
-                }
-                __syncthreads();
-            }
+        bool ok = true;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            if (!in[c]) continue;
+            const int x = 2 * i + (c ^ flip), off = c ^ flip;
+            const float* ps = sps[c ^ 1];
+            const bool hl = x > 0, hr = x + 1 < w, hu = y > 0, hd = y + 1 < h;
+            const bool good = sor_setup(px[c], inv[c] + e, np, a[c].ps, hl, hl ? ps[e - 1 + off] : 0.0f, hr, hr ? ps[e + off] : 0.0f,
+                                        hu, hu ? ps[e - pw] : 0.0f, hd, hd ? ps[e + pw] : 0.0f, a[c].a11, a[c].a12, a[c].a22,
+                                        a[c].b1, a[c].b2);
+            ok = ok && good;
+        }
+        const float lo = ok ? 1.0e-24f : INFINITY;
+        for (int s = 0; s < n_sor; s++) {
+            if (in[0]) sor_update(px[0], cur[0] + e, cur[1] + e, flip, pw, inv[0] + e, np, lo, k);
+            __syncthreads();
+            if (in[1]) sor_update(px[1], cur[1] + e, cur[0] + e, flip ^ 1, pw, inv[1] + e, np, lo, k);
+            __syncthreads();
+        }
     }
     float* u = const_cast<float*>(L.u);
     float* v = const_cast<float*>(L.v);
-    for (int o = threadIdx.x; o < n; o += blockDim.x) {
-        u[o] = __fadd_rn(su_[o], sdu[o]);
-        v[o] = __fadd_rn(sv_[o], sdv[o]);
-    }
+#pragma unroll
+    for (int c = 0; c < 2; c++)
+        if (in[c]) {
+            const long long o = (long long)y * w + 2 * i + (c ^ flip);
+            u[o] = __fadd_rn(px[c].u, px[c].du);
+            v[o] = __fadd_rn(px[c].v, px[c].dv);
+        }
 }
 
 }  // namespace
@@ -504,6 +598,24 @@ __global__ void __launch_bounds__(DF_SMALL_THREADS) k_df_level_small(DfLevel L, 
 // ---------------------------------------------------------------------------
 namespace {
 constexpr double kPi = 3.14159265358979323846;
+// One blocked SOR launch, with programmatic dependence on the kernel before it.
+cudaError_t launch_sor_tb(unsigned tiles, const DfLevel& L, const DfConst& k, int S, bool early, float* out_du, float* out_dv,
+                          cudaStream_t st) {
+    cudaLaunchAttribute attr;
+    memset(&attr, 0, sizeof(attr));
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(tiles);
+    cfg.blockDim = dim3(TB_THREADS);
+    cfg.dynamicSmemBytes = TB_SMEM;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_df_sor_tb, L, k, S, early ? 1 : 0, out_du, out_dv);
+}
+
 inline unsigned df_blocks(long long n) {
     const long long b = (n + 255) / 256;
     return (unsigned)(b < 4096 ? (b > 0 ? b : 1) : 4096);
@@ -629,8 +741,10 @@ cudaError_t dm_launch_deepflow(const DmFlowPlan& q, const DmTaps& taps, const fl
         L.w = w; L.h = h; L.n = n;
         L.D = F(q.D); L.alpha = F(q.alpha); L.mc = F(q.mc); L.mu = F(q.mu); L.mv = F(q.mv);
         L.u = cu; L.v = cv; L.du = F(q.du); L.dv = F(q.dv); L.A = F(q.A); L.ps = F(q.ps);
-        if (n <= DF_SMALL_MAX) {
-            k_df_level_small<<<1, DF_SMALL_THREADS, DF_SMALL_SMEM, st>>>(L, k, q.n_fixed, q.n_sor);
+        if ((long long)((w + 1) / 2) * h <= DF_SMALL_PAIRS) {
+            // one warp per 32 pairs: fewer warps meet at the barriers sooner
+            const int threads = ((w + 1) / 2 * h + 31) / 32 * 32;
+            k_df_level_small<<<1, threads, DF_SMALL_SMEM, st>>>(L, k, q.n_fixed, q.n_sor);
             launches++;
         } else {
             const unsigned tiles = (unsigned)(((w + TB_W - 1) / TB_W) * ((h + TB_H - 1) / TB_H));
@@ -641,7 +755,7 @@ cudaError_t dm_launch_deepflow(const DmFlowPlan& q, const DmTaps& taps, const fl
                 launches++;
                 for (int j = 0; j < 2 * q.n_sor; j += TB_S) {
                     const int S = 2 * q.n_sor - j < TB_S ? 2 * q.n_sor - j : TB_S;
-                    k_df_sor_tb<<<tiles, TB_THREADS, TB_SMEM, st>>>(L, k, j & 1, S, alt_u, alt_v);
+                    if ((e = launch_sor_tb(tiles, L, k, S, j > 0, alt_u, alt_v, st)) != cudaSuccess) return e;
                     launches++;
                     float* t = L.du; L.du = alt_u; alt_u = t;
                     t = L.dv; L.dv = alt_v; alt_v = t;
