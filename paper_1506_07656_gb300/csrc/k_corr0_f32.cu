@@ -4,49 +4,74 @@
 // written to memory: only P_0(p, r) = (max_{m} C0(p, 2r+m))^lambda and its
 // argmax code.
 //
-// Tiling.  A CTA owns 32 atomic patches (8 warps x 4) and a tile of 8 x 15
-// pooled outputs, i.e. C0 at 17 rows x 32 columns of I' positions (the
-// overlap of neighbouring 3x3 windows costs 32*17/(30*16) = 13% extra
-// correlations).  Lane j of a warp owns C0 column j for its warp's 4 patches
-// and all 17 rows: 68 accumulators, held as 34 float2 pairs (patches 0,1 and
-// 2,3) so that one packed FP32x2 fma (__ffma2_rn) updates two patches: the
-// instruction issue rate, not the FMA pipes, limited the scalar version.
-// The image-2 descriptor halo (20 rows x 35 columns x 9 channels, one float
-// each: a lane's 32-bit loads fall in distinct banks; each value is paired
-// with itself in registers for the packed fmas) and the 32 patch vectors, as
-// [(dx*9+c)*4+dy][patch], are staged in shared memory by asynchronous 4-byte
-// copies (zero-filled outside the images).
+// Tiling.  A CTA owns 32 atomic patches (8 warps x 4) and a band of 8 pooled rows,
+// and walks along it in tiles of 32 pooled columns, i.e. C0 at 17 rows x 64 columns.
+// Lane j of a warp owns the C0 columns 2j and 2j + 1 of the tile for its warp's 4
+// patches and all 17 rows: 136 accumulators, held as 68 float2 pairs of neighbouring
+// columns, so that one packed FP32x2 fma (__ffma2_rn) updates two columns.  The image-2
+// descriptors of the tile are staged channel by channel, so that a pair of
+// neighbouring columns is one 8-byte load, free of bank conflicts; a second copy,
+// shifted by one column, serves the odd offsets dx.  The patch vectors are staged with
+// every value twice.  So the main loop is packed fmas and loads alone: per (dx,
+// channel) 20 + 8 loads for 272 fmas, no moves to pair operands.  The next tile is
+// staged into a second buffer meanwhile (asynchronous 4-byte copies, zero-filled
+// outside the images: a pixel's nine floats allow no wider ones).
+//
+// Work of a CTA: an equal range of the tiles in the order (patch group, band, column),
+// about one CTA per SM and at most RANGE tiles each, so that the last wave is a full
+// one (13.5 waves of whole bands took 14).  Small inputs have fewer tiles than SMs: they
+// take lower bands and 2 patches per warp (two CTAs per SM, one buffer), by the cost
+// rule at the launch.
+//
+// What bounds it: the FMA pipe and the operand reads of the packed fmas (the main loop
+// alone runs at 77 % of the pipe's rate).  Measured (start: one lane per column, patch
+// pairs packed, operands paired by moves, 13 % overlapping tiles, 46 % of the FMA peak):
+// 512x224 6.43 -> 5.20 ms (49 % of the peak in useful fmas), 256x256 2.11 -> 1.74,
+// 64x48 25.7 -> 15.2 us.  Two CTAs of 2 patches per warp throughout: 5.43 ms (all nine
+// channels unrolled); 4 patches without the second buffer: 5.45; main loop by dy
+// instead of by staged row: 5.87; 3 channels unrolled: 5.58.
 //
 // Summation order (identical to the FP32 reference): per output,
 // acc = fma(a, b, acc) over dx = 0..3, then channel c = 0..8, then dy = 0..3,
 // starting from 0, then acc * (1/16).  Terms outside either image are zero
 // and leave acc unchanged (all operands are non-negative).  The loop order
-// (dx, c) outer / dy inner lets one column of 20 halo values in registers
-// feed all 4 dy offsets of all 17 rows.
+// (dx, c) outer / dy inner lets a staged column pair feed all 4 dy offsets: staged row
+// hr goes to the output rows hr - dy.
 //
-// Epilogue: x1/16, out-of-domain positions masked to -inf, 3x3/2 max-pool
-// with the first strict maximum in scan order (row-major in the window),
-// i.e. (no NaN occurs) the smallest scan index among the positions equal to
-// the maximum.  Each lane first reduces its own column over the three rows
-// of every pooled row (maximum and the first row reaching it); the windows
-// then combine three neighbouring columns (the smallest 3 * row + column
-// among the columns reaching the maximum), odd lanes 2k+1 for pooled row i
-// and even lanes 2k for row i+1 at once, so 30 of 32 lanes produce an output.  Maxima and
-// codes are staged in shared memory, then 240 threads raise them to lambda
-// and store rows of 15 consecutive outputs.
+// Epilogue, in registers: x1/16, out-of-domain positions masked to -inf, 3x3/2
+// max-pool with the first strict maximum in scan order (row-major in the window),
+// i.e. (no NaN occurs) the smallest scan index among the positions equal to the
+// maximum.  A lane reduces each of its two columns over the three rows of every
+// pooled row (maximum and the first row reaching it), then pools column j: the left
+// column of its window is the second column of lane j - 1, and for lane 0 the last
+// column of the tile before, which the warp keeps (so tiles do not overlap).  Then the
+// power of two rows' maxima at once and coalesced stores of 32 columns.
 #include "dm_internal.cuh"
 
 namespace {
 
-constexpr int PATCHES = 32;   // per CTA
-constexpr int CROWS = 17;     // C0 rows per CTA
-constexpr int CCOLS = 32;     // C0 columns per CTA (one per lane)
-constexpr int HROWS = CROWS + 3;
-constexpr int HCOLS = CCOLS + 3;
-constexpr int PW = 15;        // pooled columns per CTA
-constexpr int PH = 8;         // pooled rows per CTA
-constexpr int HALO_N = HROWS * HCOLS * 9;
-constexpr size_t SMEM_BYTES = (size_t)HALO_N * 4 + (size_t)144 * PATCHES * 4;
+constexpr int WARPS = 8;                      // of a CTA, NP patches each
+constexpr int PWT = 32;                       // pooled columns per tile
+constexpr int HCOLS = 2 * PWT + 3;            // pixels 64 t - 2 .. 64 t + 64
+constexpr int HPITCH = 66;                    // columns of a staged row (either copy)
+constexpr int LEFT = 12;                      // a patch's column kept for the next tile: 8 maxima, their rows, padding
+constexpr int SMS = 152;
+constexpr int RANGE = 32;                     // tiles of a CTA, at most
+
+// A band of PH pooled rows, NP patches per warp.
+template <int PH, int NP>
+struct Band {
+    static constexpr int PATCHES = WARPS * NP;
+    static constexpr int CTAS_SM = NP == 2 ? 2 : 1, BUFS = NP == 2 ? 1 : 2;
+    static constexpr int CROWS = 2 * PH + 1, HROWS = CROWS + 3;
+    // floats of a channel's plane: even, and a multiple of the banks plus 10, so that the
+    // nine channels of a pixel, which the staging writes together, fall in distinct banks
+    static constexpr int PLANE = (HROWS * HPITCH - 10 + 31) / 32 * 32 + 10;
+    static constexpr int COPY = 9 * PLANE;
+    static constexpr size_t SMEM_BYTES =
+        (size_t)(BUFS * 2 * COPY + 144 * PATCHES * 2 + WARPS * NP * LEFT + 9 * HROWS) * 4;
+    static_assert(SMEM_BYTES <= 227 * 1024 && (SMEM_BYTES + 1024) * CTAS_SM <= 228 * 1024, "shared memory");
+};
 
 // 4-byte asynchronous global -> shared copy; n = 0 writes a zero and reads nothing.
 __device__ __forceinline__ void cp_async4(float* dst, const float* src, int n) {
@@ -60,170 +85,301 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return r;
 }
 
-__global__ void __launch_bounds__(256, 2)
+// The maximum of a column over the three rows of a pooled row, and 3 x the first row
+// reaching it, shifted by sh.
+__device__ __forceinline__ float col_max(float v0, float v1, float v2, int sh, uint32_t& y3) {
+    const float m = fmax3(v0, v1, v2);
+    y3 = v0 == m ? 0u : (v1 == m ? 3u << sh : 6u << sh);
+    return m;
+}
+
+template <int PH, int NP>
+__global__ void __launch_bounds__(256, Band<PH, NP>::CTAS_SM)
 k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2, float lam,
-            float* __restrict__ pooled0, unsigned char* __restrict__ amax0, const float* __restrict__ amat, int n0) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    float* halo = reinterpret_cast<float*>(smem);                          // [HROWS][HCOLS][9]
-    float* a_s = reinterpret_cast<float*>(smem + (size_t)HALO_N * 4);      // [(dx*9+c)*4+dy][patch]
+            float* __restrict__ pooled0, unsigned char* __restrict__ amax0, const float* __restrict__ amat, int n0,
+            long long units) {
+    using B = Band<PH, NP>;
+    constexpr int CROWS = B::CROWS, HROWS = B::HROWS, PLANE = B::PLANE, COPY = B::COPY, PATCHES = B::PATCHES;
+    extern __shared__ __align__(16) float sm[];
+    // a buffer: even [9][HROWS][HPITCH], column j = pixel 64 t - 2 + j, and odd, the same
+    // shifted, column j = pixel 64 t - 1 + j
+    float2* a_s = reinterpret_cast<float2*>(sm + B::BUFS * 2 * COPY);    // [(dx*9+c)*4+dy][patch], value twice
+    float* left_s = sm + B::BUFS * 2 * COPY + 144 * PATCHES * 2;         // [warp][patch][LEFT]
+    float* edge = left_s + WARPS * NP * LEFT;                            // [9][HROWS]: pixel 64 t - 3 of the first tile
 
-    const int tiles_x = (g.dw[1] + PW - 1) / PW;
-    const int rx0 = (blockIdx.x % tiles_x) * PW;
-    const int ry0 = (blockIdx.x / tiles_x) * PH;
-    const int p_base = blockIdx.y * PATCHES;      // rows: atomic patches, or the n0 vectors of amat
-    const int W2 = g.W2, H2 = g.H2;
-    const int cx0 = 2 * rx0 - 1, cy0 = 2 * ry0 - 1;     // C0 tile origin (may be -1)
+    const int W2 = g.W2, H2 = g.H2, mw = g.dw[1], mh = g.dh[1], pitch = g.pitch(1);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tiles = (mw + PWT - 1) / PWT, bands = (mh + PH - 1) / PH;
+    const long long u0 = units * blockIdx.x / gridDim.x;
+    int todo = (int)(units * (blockIdx.x + 1) / gridDim.x - u0);
+    int t = (int)(u0 % tiles), ry0 = (int)(u0 / tiles % bands) * PH, p_base = (int)(u0 / tiles / bands) * PATCHES;
+    bool load = true, edged = t > 0;                     // stage the patch vectors, form the column before the tile
+    const DmPow pr = dm_pow_setup(lam);
 
-    // image-2 halo: pixels [cx0-2, cx0+33) x [cy0-2, cy0+18), zero outside I'
-    for (int pix = tid; pix < HROWS * HCOLS; pix += 256) {
-        int hx = pix % HCOLS, hy = pix / HCOLS;
-        int x = cx0 - 2 + hx, y = cy0 - 2 + hy;
-        bool in = (x >= 0 && y >= 0 && x < W2 && y < H2);
-        const float* src = in ? d2 + ((long long)y * W2 + x) * 9 : d2;
+    // image-2 descriptors of pixels [64 t - 2, 64 t + 65) x [2 ry0 - 3, 2 ry0 - 3 + HROWS), zero
+    // outside I': a row of them is 603 consecutive floats
+    auto stage = [&](int t, int ry0, float* even) {
+        const int y0 = 2 * ry0 - 3;
+        const bool full = t > 0 && 2 * PWT * t + 2 * PWT + 1 <= W2 && y0 >= 0 && y0 + HROWS <= H2;
+        for (int q = tid; q < HCOLS * 9; q += 256) {
+            const int col = q / 9, c = q - 9 * col;
+            const int x9 = (2 * PWT * t - 2) * 9 + q;
+            const float* src = d2 + (long long)y0 * W2 * 9 + x9;
+            float* e = even + c * PLANE + col;
+            float* o = even + COPY + c * PLANE + col - 1;
+            if (full && col >= 1 && col < HPITCH) {
 #pragma unroll
-        for (int c = 0; c < 9; c++) cp_async4(halo + pix * 9 + c, src + (in ? c : 0), in ? 4 : 0);
-    }
-    // patch vectors: window [p-2, p+1]^2 of I, zero outside I (partial
-    // patches), or row p of amat (element (dy*4 + dx)*9 + c)
-    for (int k = tid; k < 144 * PATCHES; k += 256) {
-        int pl = k % PATCHES, kk = k / PATCHES;
-        int dy = kk % 4, c = (kk / 4) % 9, dx = kk / 36;
-        int p = p_base + pl;
-        const float* src = amat ? amat : d1;
-        int n = 0;
-        if (p < n0) {
-            if (amat) {
-                src = amat + (long long)p * 144 + (dy * 4 + dx) * 9 + c;
-                n = 4;
-            } else {
-                int px = 4 * (p % g.P0x) + 2, py = 4 * (p / g.P0x) + 2;
-                int x = px - 2 + dx, y = py - 2 + dy;
-                if (x < g.W1 && y < g.H1) {
-                    src = d1 + ((long long)y * g.W1 + x) * 9 + c;
-                    n = 4;
+                for (int r = 0; r < HROWS; r++) {
+                    cp_async4(e + r * HPITCH, src, 4);
+                    cp_async4(o + r * HPITCH, src, 4);
+                    src += W2 * 9;
                 }
+                continue;
+            }
+            const bool in = x9 >= 0 && x9 < W2 * 9;
+#pragma unroll 4
+            for (int r = 0; r < HROWS; r++) {
+                const int y = y0 + r;
+                const int n = in && y >= 0 && y < H2 ? 4 : 0;
+                const float* s = n ? src : d2;
+                if (col < HPITCH) cp_async4(e + r * HPITCH, s, n);
+                if (col >= 1) cp_async4(o + r * HPITCH, s, n);
+                src += W2 * 9;
             }
         }
-        cp_async4(a_s + k, src, n);
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
+    };
 
-    float2 acc01[CROWS], acc23[CROWS];
-#pragma unroll
-    for (int r = 0; r < CROWS; r++) {
-        acc01[r] = make_float2(0.0f, 0.0f);
-        acc23[r] = make_float2(0.0f, 0.0f);
-    }
+    float* left = left_s + warp * NP * LEFT;             // this warp's: the last column of the tile before
+    float* even = sm;                                    // the tile's buffer
+    if (B::BUFS == 2) stage(t, ry0, even);
 
-    const float4* a4p = reinterpret_cast<const float4*>(a_s) + warp;   // 4 patches of this warp
+    for (; todo > 0; todo--) {
+        const int cy0 = 2 * ry0 - 1;                     // first C0 row (may be -1)
+        if (B::BUFS == 1) stage(t, ry0, even);
+        if (load) {
+            // (every warp has used the vectors before: with two buffers only the barrier here says so)
+            if (B::BUFS == 2) __syncthreads();
+            // patch vectors: window [p-2, p+1]^2 of I, zero outside I (partial
+            // patches), or row p < n0 of amat (element (dy*4 + dx)*9 + c)
+            load = false;
+            for (int k = tid; k < 144 * PATCHES; k += 256) {
+                const int pl = k % PATCHES, kk = k / PATCHES;
+                const int dy = kk % 4, c = (kk / 4) % 9, dx = kk / 36;
+                const int p = p_base + pl;
+                const float* src = amat ? amat : d1;
+                int n = 0;
+                if (p < n0) {
+                    if (amat) {
+                        src = amat + (long long)p * 144 + (dy * 4 + dx) * 9 + c;
+                        n = 4;
+                    } else {
+                        const int x = 4 * (p % g.P0x) + dx, y = 4 * (p / g.P0x) + dy;
+                        if (x < g.W1 && y < g.H1) {
+                            src = d1 + ((long long)y * g.W1 + x) * 9 + c;
+                            n = 4;
+                        }
+                    }
+                }
+                cp_async4(&a_s[k].x, src, n);
+                cp_async4(&a_s[k].y, src, n);
+            }
+        }
+        if (edged)
+            for (int k = tid; k < 9 * HROWS; k += 256) {
+                const int c = k / HROWS, y = cy0 - 2 + k % HROWS;
+                const bool in = y >= 0 && y < H2;
+                cp_async4(edge + k, in ? d2 + ((long long)y * W2 + 2 * PWT * t - 3) * 9 + c : d2, in ? 4 : 0);
+            }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+
+        // the tile after this one is staged while this one is computed
+        int tn = t + 1, yn = ry0;
+        if (tn == tiles) {
+            tn = 0;
+            yn = ry0 + PH < mh ? ry0 + PH : 0;
+        }
+        if (B::BUFS == 2 && todo > 1) stage(tn, yn, even == sm ? sm + 2 * COPY : sm);
+
+        if (edged) {
+            edged = false;
+            // the first window needs the column before the tile: lane r computes its row r
+            const int r = lane < CROWS ? lane : CROWS - 1;
+            float sv[NP] = {};
 #pragma unroll 1
-    for (int dx = 0; dx < 4; dx++) {
+            for (int k = 0; k < 36; k++) {
+                const int dx = k / 9, c = k - 9 * dx;
+                const float* hp = dx == 0 ? edge + c * HROWS + r : even + c * PLANE + r * HPITCH + dx - 1;
+                const int step = dx == 0 ? 1 : HPITCH;
+                const float2* ap = a_s + warp * NP + k * 4 * PATCHES;
+#pragma unroll
+                for (int dy = 0; dy < 4; dy++) {
+                    const float h = hp[dy * step];
+#pragma unroll
+                    for (int q = 0; q < NP; q++) sv[q] = __fmaf_rn(ap[dy * PATCHES + q].x, h, sv[q]);
+                }
+            }
+            const bool in = lane < CROWS && cy0 + lane >= 0 && cy0 + lane < H2;
+#pragma unroll
+            for (int q = 0; q < NP; q++) {
+                const float v = in ? __fmul_rn(sv[q], 0.0625f) : -INFINITY;
+                const int r3 = 2 * (lane & 7);           // lane i: pooled row i
+                const float v0 = __shfl_sync(0xffffffffu, v, r3), v1 = __shfl_sync(0xffffffffu, v, r3 + 1);
+                const float v2 = __shfl_sync(0xffffffffu, v, r3 + 2);
+                uint32_t y3;
+                const float m = col_max(v0, v1, v2, 0, y3);
+                y3 = __reduce_or_sync(0xffffffffu, y3 << (4 * (lane & 7)));
+                if (lane < PH) left[q * LEFT + lane] = m;
+                if (lane == 8) left[q * LEFT + 8] = __uint_as_float(y3);
+            }
+            __syncwarp();
+        }
+
+        float2 acc[NP][CROWS];
+#pragma unroll
+        for (int q = 0; q < NP; q++)
+#pragma unroll
+            for (int r = 0; r < CROWS; r++) acc[q][r] = make_float2(0.0f, 0.0f);
+        const float4* ap = reinterpret_cast<const float4*>(a_s) + warp * (NP / 2);      // 2 patches of this warp, each value twice
 #pragma unroll 1
-        for (int c = 0; c < 9; c++) {
-            float h[HROWS];
+        for (int dx = 0; dx < 4; dx++) {
+            const float2* hp = reinterpret_cast<const float2*>((dx & 1) ? even + COPY : even) + lane + (dx >> 1);
+#pragma unroll 1
+            for (int c = 0; c < 9; c++) {
+                float2 av[4][NP];
 #pragma unroll
-            for (int r = 0; r < HROWS; r++) h[r] = halo[(r * HCOLS + lane + dx) * 9 + c];
+                for (int dy = 0; dy < 4; dy++)
 #pragma unroll
-            for (int dy = 0; dy < 4; dy++) {
-                float4 a = a4p[((dx * 9 + c) * 4 + dy) * (PATCHES / 4)];
-                float2 a01 = make_float2(a.x, a.y), a23 = make_float2(a.z, a.w);
+                for (int q = 0; q < NP; q += 2) {
+                    const float4 a = ap[dy * (PATCHES / 2) + q / 2];
+                    av[dy][q] = make_float2(a.x, a.y);
+                    av[dy][q + 1] = make_float2(a.z, a.w);
+                }
+                // a staged row at a time: row hr feeds output row hr - dy with dy = 0..3, so each output
+                // row gets its four in order and a value is dead as soon as it is used
+#pragma unroll
+                for (int hr = 0; hr < HROWS; hr++) {
+                    const float2 h = hp[hr * (HPITCH / 2)];
+#pragma unroll
+                    for (int dy = 0; dy < 4; dy++) {
+                        const int r = hr - dy;
+                        if (r < 0 || r >= CROWS) continue;
+#pragma unroll
+                        for (int q = 0; q < NP; q++) acc[q][r] = __ffma2_rn(av[dy][q], h, acc[q][r]);
+                    }
+                }
+                hp += PLANE / 2;
+                ap += 4 * (PATCHES / 2);
+            }
+        }
+        if (B::BUFS == 1) __syncthreads();   // the next tile's descriptors may be staged
+
+        const int x = 2 * (PWT * t + lane), rx = PWT * t + lane;
+        const bool inner = 2 * PWT * (t + 1) <= W2 && cy0 >= 0 && cy0 + CROWS <= H2;
+        const long long pstride = (long long)mh * pitch;
+#pragma unroll
+        for (int q = 0; q < NP; q++) {
+            float2* v = acc[q];
+#pragma unroll
+            for (int r = 0; r < CROWS; r++) v[r] = __fmul2_rn(v[r], make_float2(0.0625f, 0.0625f));
+            if (!inner) {
 #pragma unroll
                 for (int r = 0; r < CROWS; r++) {
-                    const float2 hh = make_float2(h[r + dy], h[r + dy]);
-                    acc01[r] = __ffma2_rn(a01, hh, acc01[r]);
-                    acc23[r] = __ffma2_rn(a23, hh, acc23[r]);
+                    const bool rin = cy0 + r >= 0 && cy0 + r < H2;
+                    if (!(rin && x < W2)) v[r].x = -INFINITY;
+                    if (!(rin && x + 1 < W2)) v[r].y = -INFINITY;
                 }
             }
+            // the second column's maxima go to the lane on the right, lane 31's to the next tile
+            float right[PH], before[PH];
+            uint32_t yr = 0;
+#pragma unroll
+            for (int i = 0; i < PH; i++) {
+                uint32_t y3;
+                right[i] = col_max(v[2 * i].y, v[2 * i + 1].y, v[2 * i + 2].y, 4 * i, y3);
+                yr |= y3;
+            }
+#pragma unroll
+            for (int i = 0; i < PH; i++) before[i] = __shfl_up_sync(0xffffffffu, right[i], 1);
+            uint32_t yb = __shfl_up_sync(0xffffffffu, yr, 1);
+            float* lq = left + q * LEFT;
+            if (lane == 0) {
+#pragma unroll
+                for (int i = 0; i < PH; i++) before[i] = t > 0 ? lq[i] : -INFINITY;
+                yb = __float_as_uint(lq[8]);
+            }
+            __syncwarp();
+            if (lane == 31) {
+#pragma unroll
+                for (int i = 0; i < PH; i++) lq[i] = right[i];
+                lq[8] = __uint_as_float(yr);
+            }
+            auto pool = [&](int i, int& code) -> float {
+                uint32_t ym;
+                const float mid = col_max(v[2 * i].x, v[2 * i + 1].x, v[2 * i + 2].x, 0, ym);
+                const float best = fmax3(before[i], mid, right[i]);
+                const int k0 = before[i] == best ? (int)((yb >> (4 * i)) & 15u) : 15;
+                const int k1 = mid == best ? (int)ym + 1 : 15;
+                const int k2 = right[i] == best ? (int)((yr >> (4 * i)) & 15u) + 2 : 15;
+                code = min(k0, min(k1, k2));
+                return best;
+            };
+            const int p = p_base + NP * warp + q;
+            const bool st = rx < mw && p < n0;
+            long long o = p * pstride + (long long)ry0 * pitch + rx;
+#pragma unroll
+            for (int i = 0; i < PH; i += 2) {
+                int ca, cb;
+                const float va = pool(i, ca), vb = pool(i + 1, cb);
+                const bool out0 = st && ry0 + i < mh, out1 = st && ry0 + i + 1 < mh;
+                // (lanes without an output evaluate the power of 1)
+                const float2 pw = dm_powf2(make_float2(out0 ? va : 1.0f, out1 ? vb : 1.0f), pr);
+                if (out0) {
+                    pooled0[o] = pw.x;
+                    amax0[o] = (unsigned char)ca;
+                }
+                if (out1) {
+                    pooled0[o + pitch] = pw.y;
+                    amax0[o + pitch] = (unsigned char)cb;
+                }
+                o += 2 * pitch;
+            }
         }
+        if (tn == 0 && yn == 0) p_base += PATCHES, load = true;
+        t = tn;
+        ry0 = yn;
+        if (B::BUFS == 2) even = even == sm ? sm + 2 * COPY : sm;
     }
-    __syncthreads();   // halo and patch vectors are no longer needed: reuse the space
+}
 
-    float* best_s = reinterpret_cast<float*>(smem);                                  // [32][PH][PW]
-    unsigned char* code_s = smem + (size_t)PATCHES * PH * PW * 4;                    // [32][PH][PW]
-    const int cx = cx0 + lane;
-    const bool col_in = (cx >= 0 && cx < W2);
-    const bool odd = lane & 1;
-    const bool writer = lane < 2 * PW;             // lane 2k+1: column k of row i; lane 2k: column k of row i+1
-    const int row_sh = odd ? 0 : 4;                // this lane's pooled row (i or i+1) in a packed pair
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        float v[CROWS];
-#pragma unroll
-        for (int r = 0; r < CROWS; r++) {
-            float a = (q == 0) ? acc01[r].x : (q == 1) ? acc01[r].y : (q == 2) ? acc23[r].x : acc23[r].y;
-            int cy = cy0 + r;
-            v[r] = (col_in && cy >= 0 && cy < H2) ? __fmul_rn(a, 0.0625f) : -INFINITY;
-        }
-        // this column's maximum over the rows 2i..2i+2 of each pooled row i,
-        // and 3 x its first row reaching it, packed 4 bits per pooled row
-        float cm[PH];
-        uint32_t cyp = 0;
-#pragma unroll
-        for (int i = 0; i < PH; i++) {
-            cm[i] = fmax3(v[2 * i], v[2 * i + 1], v[2 * i + 2]);
-            const uint32_t y3 = v[2 * i] == cm[i] ? 0u : (v[2 * i + 1] == cm[i] ? 3u : 6u);
-            cyp |= y3 << (4 * i);
-        }
-        // the neighbours' columns: x0 | x1 | x2 of the window this lane pools
-        const uint32_t cyx = __shfl_xor_sync(0xffffffffu, cyp, 1);
-        const uint32_t cy1 = __shfl_down_sync(0xffffffffu, cyp, 1);
-        const uint32_t cy2 = __shfl_down_sync(0xffffffffu, cyp, 2);
-        const uint32_t y0p = odd ? cyx : cyp, y1p = odd ? cyp : cyx, y2p = odd ? cy1 : cy2;
-        const int pl = warp * 4 + q;
-#pragma unroll
-        for (int i = 0; i < PH; i += 2) {
-            const float r = __shfl_xor_sync(0xffffffffu, odd ? cm[i + 1] : cm[i], 1);
-            const float d1v = __shfl_down_sync(0xffffffffu, cm[i], 1);
-            const float d2v = __shfl_down_sync(0xffffffffu, cm[i + 1], 2);
-            const float x0 = odd ? r : cm[i + 1];
-            const float x1 = odd ? cm[i] : r;
-            const float x2 = odd ? d1v : d2v;
-            const float best = fmax3(x0, x1, x2);
-            const int sh = 4 * i + row_sh;
-            const int k0 = x0 == best ? (int)((y0p >> sh) & 15u) : 15;
-            const int k1 = x1 == best ? (int)((y1p >> sh) & 15u) + 1 : 15;
-            const int k2 = x2 == best ? (int)((y2p >> sh) & 15u) + 2 : 15;
-            const int code = min(k0, min(k1, k2));
-            if (writer) {
-                const int e = (pl * PH + i + (odd ? 0 : 1)) * PW + (lane >> 1);
-                best_s[e] = best;
-                code_s[e] = (unsigned char)code;
-            }
-        }
-    }
-    __syncthreads();
-    // 240 threads raise the staged maxima to lambda: thread t keeps column
-    // t % 15 and pooled row (t / 15) % 8, and takes every second patch from
-    // t / 120, two patches per packed evaluation (bit-identical to dm_powf
-    // lane by lane); consecutive threads store consecutive outputs of a row
-    if (tid < 16 * PW) {
-        const int kk = tid % PW, u0 = tid / PW;
-        const int rx = rx0 + kk, ry = ry0 + (u0 % PH);
-        const int mw = g.dw[1], mh = g.dh[1];
-        const DmPow pr = dm_pow_setup(lam);
-        if (rx < mw && ry < mh) {
-            const int pl0 = u0 / PH;
-            const long long pstride = (long long)mh * g.pitch(1);
-            const long long o0 = ((long long)(p_base + pl0) * mh + ry) * g.pitch(1) + rx;
-#pragma unroll 2
-            for (int j = 0; j < PATCHES / 2; j += 2) {
-                const int e = tid + j * 16 * PW;
-                const float2 v = dm_powf2(make_float2(best_s[e], best_s[e + 16 * PW]), pr);
-                const int p = p_base + pl0 + 2 * j;
-                const long long o = o0 + 2 * j * pstride;
-                if (p < n0) {
-                    pooled0[o] = v.x;
-                    amax0[o] = code_s[e];
-                }
-                if (p + 2 < n0) {
-                    pooled0[o + 2 * pstride] = v.y;
-                    amax0[o + 2 * pstride] = code_s[e + 16 * PW];
-                }
-            }
-        }
-    }
+template <int PH, int NP>
+long long band_units(const DmGeom& g, int n_rows) {
+    constexpr int P = Band<PH, NP>::PATCHES;
+    return (long long)((n_rows + P - 1) / P) * ((g.dh[1] + PH - 1) / PH) * ((g.dw[1] + PWT - 1) / PWT);
+}
+
+// The time of a form: tiles of the busiest SM, each its C0 rows and what costs about four
+// more of them besides, for the patches of a CTA; a quarter more where the CTAs of small
+// inputs begin inside a band, at a window that needs a column of its own.
+template <int PH, int NP>
+long long band_cost(const DmGeom& g, int n_rows) {
+    const long long c = (band_units<PH, NP>(g, n_rows) + SMS - 1) / SMS * (2 * PH + 5) * NP;
+    return NP == 2 && g.dw[1] > PWT ? c + c / 4 : c;
+}
+
+template <int PH, int NP>
+cudaError_t launch_band(const DmGeom& g, const float* d1, const float* d2, float lam, float* pooled0, unsigned char* amax0,
+                        cudaStream_t st, const float* amat, int n_rows) {
+    using B = Band<PH, NP>;
+    static std::atomic<unsigned long long> smem_done{0};   // > 48 KB dynamic shared memory opted in, per device
+    cudaError_t e = dm_smem_opt_in(reinterpret_cast<const void*>(k_corr0_f32<PH, NP>), (int)B::SMEM_BYTES, smem_done);
+    if (e != cudaSuccess) return e;
+    const long long units = band_units<PH, NP>(g, n_rows), slots = SMS * B::CTAS_SM;
+    const long long waves = (units + slots * RANGE - 1) / (slots * RANGE);
+    const long long grid = units < slots ? units : slots * waves;
+    k_corr0_f32<PH, NP><<<(unsigned)grid, 256, B::SMEM_BYTES, st>>>(g, d1, d2, lam, pooled0, amax0, amat, n_rows, units);
+    dm_count_launches(1);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -231,13 +387,12 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
 cudaError_t dm_launch_corr0_f32(const DmGeom& g, const float* d1, const float* d2, float lam, float* pooled0,
                                 unsigned char* amax0, cudaStream_t st, const float* amat, int n_rows) {
     if (n_rows < 0) n_rows = g.P0x * g.P0y;
-    int tiles = ((g.dw[1] + PW - 1) / PW) * ((g.dh[1] + PH - 1) / PH);
-    int pblocks = (n_rows + PATCHES - 1) / PATCHES;
-    dim3 grid(tiles, pblocks);
-    static std::atomic<unsigned long long> smem_done{0};   // > 48 KB dynamic shared memory opted in, per device
-    cudaError_t e = dm_smem_opt_in(reinterpret_cast<const void*>(k_corr0_f32), (int)SMEM_BYTES, smem_done);
-    if (e != cudaSuccess) return e;
-    k_corr0_f32<<<grid, 256, SMEM_BYTES, st>>>(g, d1, d2, lam, pooled0, amax0, amat, n_rows);
-    dm_count_launches(1);
-    return cudaGetLastError();
+    // The form with the shortest way: bands of 8 rows do the least extra work (17 C0 rows for
+    // 16, against 9 for 8 and 5 for 4) and are taken by all but inputs of few tiles, whose
+    // time is that of the busiest SM (64x48: 15.2 us with bands of 2, 29.5 with 8; 128x96: 83 us
+    // with 8 rows and 4 patches, 88 with 2 patches).
+    const long long c8 = band_cost<8, 4>(g, n_rows), c4 = band_cost<4, 2>(g, n_rows), c2 = band_cost<2, 2>(g, n_rows);
+    if (c8 <= c4 && c8 <= c2) return launch_band<8, 4>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows);
+    if (c4 <= c2) return launch_band<4, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows);
+    return launch_band<2, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows);
 }
