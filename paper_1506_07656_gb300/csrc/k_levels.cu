@@ -101,25 +101,6 @@ constexpr long long LEVEL_WAIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
 // additions, every step correctly rounded per lane) costs 3 instructions per
 // column and step.
 template <bool COMP, bool DIV3>
-__device__ __forceinline__ float2 avg_pair4(float2 x0, float2 x1, float2 x2, float2 x3, float w) {
-    float2 sv = x0;
-    if constexpr (COMP) {
-        float2 cp, err;
-        // first step: the compensation starts as its error term (0 + err = err;
-        // a -0 there would only meet s + (+-0) = s at the end)
-        dm_two_sum2(sv, x1, cp);
-        dm_two_sum2(sv, x2, err);
-        cp = __fadd2_rn(cp, err);
-        dm_two_sum2(sv, x3, err);
-        cp = __fadd2_rn(cp, err);
-        sv = __fadd2_rn(sv, cp);
-    } else {
-        sv = __fadd2_rn(__fadd2_rn(__fadd2_rn(sv, x1), x2), x3);
-    }
-    return DIV3 ? make_float2(__fdiv_rn(sv.x, 3.0f), __fdiv_rn(sv.y, 3.0f)) : __fmul2_rn(sv, make_float2(w, w));
-}
-
-template <bool COMP, bool DIV3>
 __device__ __forceinline__ float4 avg_group(const float* lt, const float* lb, const float* rt, const float* rb, float w) {
     const float4 a0 = *reinterpret_cast<const float4*>(lt), b0 = *reinterpret_cast<const float4*>(lt + 4);
     const float4 a1 = *reinterpret_cast<const float4*>(lb), b1 = *reinterpret_cast<const float4*>(lb + 4);
