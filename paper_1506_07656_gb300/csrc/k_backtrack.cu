@@ -35,6 +35,8 @@
 // A patch's best tuple is output iff it also wins its cell of I'.
 #include "dm_internal.cuh"
 
+#include <cooperative_groups.h>
+
 #include <memory>
 
 namespace {
@@ -388,17 +390,31 @@ __device__ __forceinline__ void bt_expand_body(const BtArgs& a, int l) {
 template <int MODE, bool K64>
 __global__ void k_bt_expand(BtArgs a, int l) { bt_expand_body<MODE, K64>(a, l); }
 
-// Reciprocal verification and compaction in atomic-patch order (one block).
+// Reciprocal verification and compaction in atomic-patch order: one cluster of
+// RECIP_CTAS CTAs per pair.  Warp w of the cluster owns a run of consecutive patches
+// (whole warps of them, so the reads of BestAt are coalesced); it counts its survivors,
+// the CTAs exchange their counts through distributed shared memory, and each warp
+// writes its survivors behind those of the warps before it.
+//
+// What bounds it: the latency of two dependent loads per patch and pass (a patch's key,
+// then the key of the cell that it points to).  1024x436 (27904 patches): 83 -> 13 us;
+// one CTA, its threads on runs of 28 patches each, before.
+constexpr int RECIP_CTAS = 8, RECIP_THREADS = 1024;
+
 __device__ __forceinline__ void reciprocal_body(const BtArgs& a, dm_match_t* __restrict__ out, int capacity,
                                                 int* __restrict__ d_count) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
     const DmGeom& g = a.g;
     const int n0 = g.npatch(0);
     const int CW = (g.W2 + 3) >> 2;
-    const int chunk = (n0 + blockDim.x - 1) / blockDim.x;
-    const int p0 = threadIdx.x * chunk;
-    const int p1 = min(n0, p0 + chunk);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rank = (int)cluster.block_rank();
+    constexpr int WARPS = RECIP_THREADS / 32;
+    const int run = ((n0 + 31) / 32 + RECIP_CTAS * WARPS - 1) / (RECIP_CTAS * WARPS) * 32;   // patches of a warp
+    const long long first = (long long)(rank * WARPS + warp) * run;
+    const int p0 = (int)min((long long)n0, first), p1 = min(n0, p0 + run);
     __shared__ int warp_sums[32];
-    __shared__ int total;
+    __shared__ int total;                               // this CTA's survivors
 
     auto survives = [&](int p, int& tx, int& ty, float& s) -> bool {
         unsigned long long kp = a.bestP[p];
@@ -413,60 +429,59 @@ __device__ __forceinline__ void reciprocal_body(const BtArgs& a, dm_match_t* __r
         return (kq >> 32) == (kp >> 32) && qidx == (unsigned int)p * 16u + (unsigned int)((ty & 3) * 4 + (tx & 3));
     };
 
-    int mine = 0;
-    for (int p = p0; p < p1; p++) {
+    int mine = 0;                                       // the warp's survivors
+    for (int p = p0 + lane; p - lane < p1; p += 32) {
         int tx, ty;
         float s;
-        mine += survives(p, tx, ty, s) ? 1 : 0;
+        mine += __popc(__ballot_sync(0xffffffffu, p < p1 && survives(p, tx, ty, s)));
     }
-    // block exclusive scan of `mine`
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) warp_sums[warp] = incl;
+    if (lane == 0) warp_sums[warp] = mine;
     __syncthreads();
-    if (warp == 0) {
-        int nw = blockDim.x >> 5;
-        int w = lane < nw ? warp_sums[lane] : 0;
+    if (warp == 0) {                                    // exclusive scan over the CTA's warps
+        const int w = warp_sums[lane];
         int wi = w;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             int v = __shfl_up_sync(0xffffffffu, wi, o);
             if (lane >= o) wi += v;
         }
-        if (lane < nw) warp_sums[lane] = wi - w;
+        warp_sums[lane] = wi - w;
         if (lane == 31) total = wi;
     }
-    __syncthreads();
-    int pos = warp_sums[warp] + incl - mine;
-    for (int p = p0; p < p1; p++) {
+    cluster.sync();
+    int before = 0, all = 0;
+    for (int r = 0; r < RECIP_CTAS; r++) {
+        const int n = *cluster.map_shared_rank(&total, r);
+        before += r < rank ? n : 0;
+        all += n;
+    }
+    cluster.sync();                                     // no CTA leaves while its count may be read
+    int pos = before + warp_sums[warp];
+    for (int p = p0 + lane; p - lane < p1; p += 32) {
         int tx, ty;
         float s;
-        if (survives(p, tx, ty, s)) {
-            if (pos < capacity) {
-                dm_match_t m;
-                m.x1 = (float)(4 * (p % g.P0x) + 2);
-                m.y1 = (float)(4 * (p / g.P0x) + 2);
-                m.x2 = (float)tx;
-                m.y2 = (float)ty;
-                m.score = s;
-                out[pos] = m;
-            }
-            pos++;
+        const bool keep = p < p1 && survives(p, tx, ty, s);
+        const unsigned int kept = __ballot_sync(0xffffffffu, keep);
+        const int at = pos + __popc(kept & ((1u << lane) - 1u));
+        if (keep && at < capacity) {
+            dm_match_t m;
+            m.x1 = (float)(4 * (p % g.P0x) + 2);
+            m.y1 = (float)(4 * (p / g.P0x) + 2);
+            m.x2 = (float)tx;
+            m.y2 = (float)ty;
+            m.score = s;
+            out[at] = m;
         }
+        pos += __popc(kept);
     }
-    if (threadIdx.x == 0) {
-        *d_count = total;
-        if (total > capacity) atomicOr(&a.hdr->status, DM_DEV_OUTPUT_OVERFLOW);
+    if (rank == 0 && threadIdx.x == 0) {
+        *d_count = all;
+        if (all > capacity) atomicOr(&a.hdr->status, DM_DEV_OUTPUT_OVERFLOW);
     }
 }
 
-__global__ void __launch_bounds__(1024) k_reciprocal(BtArgs a, dm_match_t* __restrict__ out, int capacity,
-                                                     int* __restrict__ d_count) {
+__global__ void __cluster_dims__(RECIP_CTAS, 1, 1) __launch_bounds__(RECIP_THREADS)
+k_reciprocal(BtArgs a, dm_match_t* __restrict__ out, int capacity, int* __restrict__ d_count) {
     reciprocal_body(a, out, capacity, d_count);
 }
 
@@ -692,7 +707,7 @@ int sm_count() {
 }
 
 // Cross-pair form: the pairs of a wave of the batched form in one launch per
-// step, pair blockIdx.y (blockIdx.x for the reciprocal step), its arguments in
+// step, pair blockIdx.y (a cluster of blockIdx.x for the reciprocal step), its arguments in
 // the kernel parameters (a captured graph replays them as they were).  Step s
 // of the backtracking works on level lvl[j] = L_j - s of pair j.
 struct BtBatch {
@@ -721,8 +736,10 @@ __global__ void k_bt_expand_b(const __grid_constant__ BtBatch B) {
     bt_expand_body<BT_EXACT, K64>(B.a[blockIdx.y], B.lvl[blockIdx.y]);
 }
 
-__global__ void __launch_bounds__(1024) k_reciprocal_b(const __grid_constant__ BtBatch B) {
-    reciprocal_body(B.a[blockIdx.x], B.out[blockIdx.x], B.capacity[blockIdx.x], B.count[blockIdx.x]);
+__global__ void __cluster_dims__(RECIP_CTAS, 1, 1) __launch_bounds__(RECIP_THREADS)
+k_reciprocal_b(const __grid_constant__ BtBatch B) {
+    const int j = blockIdx.x / RECIP_CTAS;
+    reciprocal_body(B.a[j], B.out[j], B.capacity[j], B.count[j]);
 }
 
 }  // namespace
@@ -740,7 +757,7 @@ cudaError_t dm_launch_backtrack(const DmGeom& g, const dm_pyramid& py, const DmB
         return cudaGetLastError();
     }
     launch_steps<BT_EXACT>(a, grid, st);
-    k_reciprocal<<<1, 1024, 0, st>>>(a, out, capacity, d_count);
+    k_reciprocal<<<RECIP_CTAS, RECIP_THREADS, 0, st>>>(a, out, capacity, d_count);
     dm_count_launches(2 * g.L);
     return cudaGetLastError();
 }
@@ -800,7 +817,7 @@ cudaError_t dm_launch_backtrack_star(const DmGeom& g, const dm_pyramid& py, cons
         }
         k_bt_expand<BT_STAR, false><<<grid, BT_BLOCK, 0, st>>>(a, l);
     }
-    k_reciprocal<<<1, 1024, 0, st>>>(a, out, capacity, d_count);
+    k_reciprocal<<<RECIP_CTAS, RECIP_THREADS, 0, st>>>(a, out, capacity, d_count);
     dm_count_launches(4 * g.L + 1);
     return cudaGetLastError();
 }
@@ -813,7 +830,7 @@ cudaError_t dm_launch_reciprocal(const DmGeom& g, unsigned long long* bestP, uns
     a.bestP = bestP;
     a.bestQ = bestQ;
     a.hdr = hdr;
-    k_reciprocal<<<1, 1024, 0, st>>>(a, out, capacity, d_count);
+    k_reciprocal<<<RECIP_CTAS, RECIP_THREADS, 0, st>>>(a, out, capacity, d_count);
     dm_count_launches(1);
     return cudaGetLastError();
 }
@@ -894,7 +911,7 @@ cudaError_t dm_launch_backtrack_batch(const dm_pyramid* const* pys, const DmBtLa
             launches++;
         }
     }
-    k_reciprocal_b<<<n, 1024, 0, st>>>(all);
+    k_reciprocal_b<<<n * RECIP_CTAS, RECIP_THREADS, 0, st>>>(all);
     dm_count_launches(launches + 1);
     return cudaGetLastError();
 }
