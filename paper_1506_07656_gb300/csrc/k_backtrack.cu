@@ -278,13 +278,41 @@ __global__ void k_star_prepare(BtArgs a, int lvl) {
 }
 
 template <bool K64>
-__device__ __forceinline__ void bt_prepare_body(const BtArgs& a, int lvl, long long n_top) {
-    const unsigned long long n_prev = (lvl + 1 == a.g.L) ? (unsigned long long)n_top : a.hdr->count[lvl + 1];
-    clear_table<K64>(a, lvl, (n_prev * HT_SLOTS_PER_PREV + 31ull) & ~31ull);
+__device__ __forceinline__ void bt_prepare_body(const BtArgs& a, int lvl) {
+    clear_table<K64>(a, lvl, ((unsigned long long)a.hdr->count[lvl + 1] * HT_SLOTS_PER_PREV + 31ull) & ~31ull);
+}
+
+// The start of a pair's backtracking in one launch: the step's part of the header (status
+// word, counts, table sizes; pyr_status belongs to the pyramid step that ran before),
+// unless the tuples go to another pair's keys (the invariant form) the BestAt / BestAt'
+// keys, and the first table, whose size the top level gives.
+template <bool K64>
+__device__ __forceinline__ void bt_begin_body(const BtArgs& a, bool keys) {
+    const DmGeom& g = a.g;
+    const int lvl = g.L - 1;
+    if (blockIdx.x == 0) {
+        for (unsigned int i = threadIdx.x; i < DM_MAXL + 2; i += blockDim.x) {
+            a.hdr->count[i] = 0u;
+            if ((int)i != lvl || lvl < 1) a.hdr->cap[i] = 0u;    // (clear_table sets the first table's)
+        }
+        if (threadIdx.x == 0) a.hdr->status = 0;
+    }
+    if (keys) {
+        const long long n0 = g.npatch(0), n = n0 + (long long)((g.W2 + 3) / 4) * ((g.H2 + 3) / 4);
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+            if (i < n0) a.bestP[i] = 0ull;
+            else a.bestQ[i - n0] = 0ull;
+        }
+    }
+    if (lvl >= 1)
+        clear_table<K64>(a, lvl, ((unsigned long long)g.npatch(g.L) * g.dsize(g.L) * HT_SLOTS_PER_PREV + 31ull) & ~31ull);
 }
 
 template <bool K64>
-__global__ void k_bt_prepare(BtArgs a, int lvl, long long n_top) { bt_prepare_body<K64>(a, lvl, n_top); }
+__global__ void k_bt_begin(BtArgs a, int keys) { bt_begin_body<K64>(a, keys != 0); }
+
+template <bool K64>
+__global__ void k_bt_prepare(BtArgs a, int lvl) { bt_prepare_body<K64>(a, lvl); }
 
 // Expansion of the top level: every position of every existing top patch.
 template <int MODE, bool K64>
@@ -636,11 +664,12 @@ __global__ void k_star_insert(BtArgs a, int l) {
 }
 
 template <int MODE, bool K64>
-void launch_steps_k(const BtArgs& a, int grid, cudaStream_t st) {
+void launch_steps_k(const BtArgs& a, int grid, int keys, cudaStream_t st) {
     const DmGeom& g = a.g;
     const long long n_top = (long long)g.npatch(g.L) * g.dsize(g.L);
     for (int l = g.L; l >= 1; l--) {
-        if (l - 1 >= 1) k_bt_prepare<K64><<<grid, BT_BLOCK, 0, st>>>(a, l - 1, n_top);
+        if (l == g.L) k_bt_begin<K64><<<grid, BT_BLOCK, 0, st>>>(a, keys);
+        else if (l - 1 >= 1) k_bt_prepare<K64><<<grid, BT_BLOCK, 0, st>>>(a, l - 1);
         if (l == g.L) {
             long long nb = (n_top + BT_BLOCK - 1) / BT_BLOCK;
             k_bt_expand_top<MODE, K64><<<(unsigned)(nb < grid ? nb : grid), BT_BLOCK, 0, st>>>(a);
@@ -652,8 +681,10 @@ void launch_steps_k(const BtArgs& a, int grid, cudaStream_t st) {
 
 template <int MODE>
 void launch_steps(const BtArgs& a, int grid, cudaStream_t st) {
-    if (a.g.key64) launch_steps_k<MODE, true>(a, grid, st);
-    else launch_steps_k<MODE, false>(a, grid, st);
+    const int keys = MODE != BT_RECT;
+    if (a.g.key64) launch_steps_k<MODE, true>(a, grid, keys, st);
+    else launch_steps_k<MODE, false>(a, grid, keys, st);
+    dm_count_launches(a.g.L == 1 ? 2 : 2 * a.g.L - 1);
 }
 
 }  // namespace
@@ -683,22 +714,6 @@ BtArgs make_bt_args(const DmGeom& g, const dm_pyramid& py, const DmBtLayout& bl,
     return a;
 }
 
-// Clear the backtracking part of the header (status word, counts, table
-// sizes; pyr_status belongs to the pyramid step that ran before) and, unless
-// the tuples go to another pair's keys (rect), the BestAt / BestAt' keys.
-cudaError_t clear_bt(const BtArgs& a, bool keys, cudaStream_t st) {
-    const DmGeom& g = a.g;
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(&a.hdr->status, 0, sizeof(int), st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a.hdr->count, 0, sizeof(a.hdr->count) + sizeof(a.hdr->cap), st)) != cudaSuccess) return e;
-    if (keys) {
-        if ((e = cudaMemsetAsync(a.bestP, 0, sizeof(unsigned long long) * g.npatch(0), st)) != cudaSuccess) return e;
-        size_t ncell = (size_t)((g.W2 + 3) / 4) * ((g.H2 + 3) / 4);
-        if ((e = cudaMemsetAsync(a.bestQ, 0, sizeof(unsigned long long) * ncell, st)) != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
 int sm_count() {
     int dev = 0, nsm = 148;
     cudaGetDevice(&dev);
@@ -721,9 +736,13 @@ struct BtBatch {
 static_assert(sizeof(BtBatch) < 32000, "the kernel parameters of a wave must stay below the 32 KB limit");
 
 template <bool K64>
+__global__ void k_bt_begin_b(const __grid_constant__ BtBatch B) {
+    bt_begin_body<K64>(B.a[blockIdx.y], true);
+}
+
+template <bool K64>
 __global__ void k_bt_prepare_b(const __grid_constant__ BtBatch B) {
-    const BtArgs& a = B.a[blockIdx.y];
-    bt_prepare_body<K64>(a, B.lvl[blockIdx.y] - 1, (long long)a.g.npatch(a.g.L) * a.g.dsize(a.g.L));
+    bt_prepare_body<K64>(B.a[blockIdx.y], B.lvl[blockIdx.y] - 1);
 }
 
 template <bool K64>
@@ -748,17 +767,14 @@ cudaError_t dm_launch_backtrack(const DmGeom& g, const dm_pyramid& py, const DmB
                                 dm_match_t* out, int capacity, int* d_count, cudaStream_t st, const DmRect* rect) {
     BtArgs a = make_bt_args(g, py, bl, ws);
     if (rect) a.rect = *rect;
-    cudaError_t e = clear_bt(a, !rect, st);
-    if (e != cudaSuccess) return e;
     const int grid = sm_count() * (py.tune.bt_mult > 0 ? py.tune.bt_mult : 8);
     if (rect) {
         launch_steps<BT_RECT>(a, grid, st);
-        dm_count_launches(2 * g.L - 1);
         return cudaGetLastError();
     }
     launch_steps<BT_EXACT>(a, grid, st);
     k_reciprocal<<<RECIP_CTAS, RECIP_THREADS, 0, st>>>(a, out, capacity, d_count);
-    dm_count_launches(2 * g.L);
+    dm_count_launches(1);
     return cudaGetLastError();
 }
 
@@ -848,13 +864,11 @@ cudaError_t dm_launch_backtrack_batch(const dm_pyramid* const* pys, const DmBtLa
     memset(&all, 0, sizeof(all));
     all.n = n;
     int Lmax = 0, mult = 8;
-    cudaError_t e;
     for (int j = 0; j < n; j++) {
         all.a[j] = make_bt_args(pys[j]->g, *pys[j], *bls[j], wss[j]);
         all.out[j] = outs[j];
         all.capacity[j] = caps[j];
         all.count[j] = counts[j];
-        if ((e = clear_bt(all.a[j], true, st)) != cudaSuccess) return e;
         Lmax = max(Lmax, pys[j]->g.L);
         if (pys[j]->tune.bt_mult > 0) mult = pys[j]->tune.bt_mult;
     }
@@ -881,7 +895,11 @@ cudaError_t dm_launch_backtrack_batch(const dm_pyramid* const* pys, const DmBtLa
             BtBatch& b = sub;
             int with_next = 0;
             for (int j = 0; j < b.n; j++) with_next += b.lvl[j] - 1 >= 1;
-            if (with_next == b.n) {
+            if (step == 0) {
+                if (k64) k_bt_begin_b<true><<<dim3(per, b.n), BT_BLOCK, 0, st>>>(b);
+                else k_bt_begin_b<false><<<dim3(per, b.n), BT_BLOCK, 0, st>>>(b);
+                launches++;
+            } else if (with_next == b.n) {
                 if (k64) k_bt_prepare_b<true><<<dim3(per, b.n), BT_BLOCK, 0, st>>>(b);
                 else k_bt_prepare_b<false><<<dim3(per, b.n), BT_BLOCK, 0, st>>>(b);
                 launches++;
