@@ -309,10 +309,16 @@ __device__ __forceinline__ void bt_begin_body(const BtArgs& a, bool keys) {
 }
 
 template <bool K64>
-__global__ void k_bt_begin(BtArgs a, int keys) { bt_begin_body<K64>(a, keys != 0); }
+__global__ void k_bt_begin(BtArgs a, int keys) {
+    dm_pdl_wait();
+    bt_begin_body<K64>(a, keys != 0);
+}
 
 template <bool K64>
-__global__ void k_bt_prepare(BtArgs a, int lvl) { bt_prepare_body<K64>(a, lvl); }
+__global__ void k_bt_prepare(BtArgs a, int lvl) {
+    dm_pdl_wait();
+    bt_prepare_body<K64>(a, lvl);
+}
 
 // Expansion of the top level: every position of every existing top patch.
 template <int MODE, bool K64>
@@ -338,7 +344,10 @@ __device__ __forceinline__ void bt_expand_top_body(const BtArgs& a) {
 }
 
 template <int MODE, bool K64>
-__global__ void k_bt_expand_top(BtArgs a) { bt_expand_top_body<MODE, K64>(a); }
+__global__ void k_bt_expand_top(BtArgs a) {
+    dm_pdl_wait();
+    bt_expand_top_body<MODE, K64>(a);
+}
 
 // Expansion of level l < L: the merged tuples of level l, read by scanning the
 // active part of its table in slot order.  Each warp packs the occupied slots
@@ -416,7 +425,10 @@ __device__ __forceinline__ void bt_expand_body(const BtArgs& a, int l) {
 }
 
 template <int MODE, bool K64>
-__global__ void k_bt_expand(BtArgs a, int l) { bt_expand_body<MODE, K64>(a, l); }
+__global__ void k_bt_expand(BtArgs a, int l) {
+    dm_pdl_wait();
+    bt_expand_body<MODE, K64>(a, l);
+}
 
 // Reciprocal verification and compaction in atomic-patch order: one cluster of
 // RECIP_CTAS CTAs per pair.  Warp w of the cluster owns a run of consecutive patches
@@ -510,6 +522,7 @@ __device__ __forceinline__ void reciprocal_body(const BtArgs& a, dm_match_t* __r
 
 __global__ void __cluster_dims__(RECIP_CTAS, 1, 1) __launch_bounds__(RECIP_THREADS)
 k_reciprocal(BtArgs a, dm_match_t* __restrict__ out, int capacity, int* __restrict__ d_count) {
+    dm_pdl_wait();
     reciprocal_body(a, out, capacity, d_count);
 }
 
@@ -668,13 +681,13 @@ void launch_steps_k(const BtArgs& a, int grid, int keys, cudaStream_t st) {
     const DmGeom& g = a.g;
     const long long n_top = (long long)g.npatch(g.L) * g.dsize(g.L);
     for (int l = g.L; l >= 1; l--) {
-        if (l == g.L) k_bt_begin<K64><<<grid, BT_BLOCK, 0, st>>>(a, keys);
-        else if (l - 1 >= 1) k_bt_prepare<K64><<<grid, BT_BLOCK, 0, st>>>(a, l - 1);
+        if (l == g.L) dm_launch_pdl(k_bt_begin<K64>, grid, BT_BLOCK, 0, st, a, keys);
+        else if (l - 1 >= 1) dm_launch_pdl(k_bt_prepare<K64>, grid, BT_BLOCK, 0, st, a, l - 1);
         if (l == g.L) {
             long long nb = (n_top + BT_BLOCK - 1) / BT_BLOCK;
-            k_bt_expand_top<MODE, K64><<<(unsigned)(nb < grid ? nb : grid), BT_BLOCK, 0, st>>>(a);
+            dm_launch_pdl(k_bt_expand_top<MODE, K64>, (unsigned)(nb < grid ? nb : grid), BT_BLOCK, 0, st, a);
         } else {
-            k_bt_expand<MODE, K64><<<grid, BT_BLOCK, 0, st>>>(a, l);
+            dm_launch_pdl(k_bt_expand<MODE, K64>, grid, BT_BLOCK, 0, st, a, l);
         }
     }
 }
@@ -773,7 +786,7 @@ cudaError_t dm_launch_backtrack(const DmGeom& g, const dm_pyramid& py, const DmB
         return cudaGetLastError();
     }
     launch_steps<BT_EXACT>(a, grid, st);
-    k_reciprocal<<<RECIP_CTAS, RECIP_THREADS, 0, st>>>(a, out, capacity, d_count);
+    dm_launch_pdl(k_reciprocal, RECIP_CTAS, RECIP_THREADS, 0, st, a, out, capacity, d_count);
     dm_count_launches(1);
     return cudaGetLastError();
 }
@@ -831,9 +844,9 @@ cudaError_t dm_launch_backtrack_star(const DmGeom& g, const dm_pyramid& py, cons
             k_star_prepare<<<grid, BT_BLOCK, 0, st>>>(a, l - 1);
             k_star_insert<<<grid, BT_BLOCK, 0, st>>>(a, l - 1);
         }
-        k_bt_expand<BT_STAR, false><<<grid, BT_BLOCK, 0, st>>>(a, l);
+        dm_launch_pdl(k_bt_expand<BT_STAR, false>, grid, BT_BLOCK, 0, st, a, l);
     }
-    k_reciprocal<<<RECIP_CTAS, RECIP_THREADS, 0, st>>>(a, out, capacity, d_count);
+    dm_launch_pdl(k_reciprocal, RECIP_CTAS, RECIP_THREADS, 0, st, a, out, capacity, d_count);
     dm_count_launches(4 * g.L + 1);
     return cudaGetLastError();
 }
@@ -846,7 +859,7 @@ cudaError_t dm_launch_reciprocal(const DmGeom& g, unsigned long long* bestP, uns
     a.bestP = bestP;
     a.bestQ = bestQ;
     a.hdr = hdr;
-    k_reciprocal<<<RECIP_CTAS, RECIP_THREADS, 0, st>>>(a, out, capacity, d_count);
+    dm_launch_pdl(k_reciprocal, RECIP_CTAS, RECIP_THREADS, 0, st, a, out, capacity, d_count);
     dm_count_launches(1);
     return cudaGetLastError();
 }

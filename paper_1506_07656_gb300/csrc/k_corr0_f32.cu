@@ -115,6 +115,7 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
     int t = (int)(u0 % tiles), ry0 = (int)(u0 / tiles % bands) * PH, p_base = (int)(u0 / tiles / bands) * PATCHES;
     bool load = true, edged = t > 0;                     // stage the patch vectors, form the column before the tile
     const DmPow pr = dm_pow_setup(lam);
+    dm_pdl_wait();
 
     // image-2 descriptors of pixels [64 t - 2, 64 t + 65) x [2 ry0 - 3, 2 ry0 - 3 + HROWS), zero
     // outside I': a row of them is 603 consecutive floats
@@ -377,7 +378,9 @@ cudaError_t launch_band(const DmGeom& g, const float* d1, const float* d2, float
     const long long units = band_units<PH, NP>(g, n_rows), slots = SMS * B::CTAS_SM;
     const long long waves = (units + slots * RANGE - 1) / (slots * RANGE);
     const long long grid = units < slots ? units : slots * waves;
-    k_corr0_f32<PH, NP><<<(unsigned)grid, 256, B::SMEM_BYTES, st>>>(g, d1, d2, lam, pooled0, amax0, amat, n_rows, units);
+    e = dm_launch_pdl(k_corr0_f32<PH, NP>, (unsigned)grid, 256, B::SMEM_BYTES, st, g, d1, d2, lam, pooled0, amax0, amat, n_rows,
+                      units);
+    if (e != cudaSuccess) return e;
     dm_count_launches(1);
     return cudaGetLastError();
 }

@@ -343,6 +343,7 @@ template <int TX, int TY>
 __global__ void __launch_bounds__(DESC_THREADS) k_descriptors(const float* __restrict__ img, float* __restrict__ desc, int W,
                                                               int H, Taps7 t1, Taps7 t2, Taps7 t3, float scale, float slope,
                                                               float mu) {
+    dm_pdl_wait();
     desc_tile<TX, TY>(img, desc, W, H, blockIdx.x, t1, t2, t3, scale, slope, mu);
 }
 
@@ -371,8 +372,9 @@ cudaError_t launch_fused(const DmDescParams& prm, const Taps7 t[3], const IoBatc
     for (int i = 0; i < b.n; i++) tiles = std::max(tiles, (unsigned)((b.W[i] + TX - 1) / TX) * (unsigned)((b.H[i] + TY - 1) / TY));
     if (b.n == 1) {
         if ((e = dm_smem_opt_in(reinterpret_cast<const void*>(k_descriptors<TX, TY>), smem, done)) != cudaSuccess) return e;
-        k_descriptors<TX, TY><<<tiles, DESC_THREADS, smem, st>>>(b.in[0], b.out[0], b.W[0], b.H[0], t[0], t[1], t[2], prm.scale,
-                                                                 prm.slope, prm.mu);
+        e = dm_launch_pdl(k_descriptors<TX, TY>, tiles, DESC_THREADS, smem, st, b.in[0], b.out[0], b.W[0], b.H[0], t[0], t[1], t[2],
+                          prm.scale, prm.slope, prm.mu);
+        if (e != cudaSuccess) return e;
     } else {
         if ((e = dm_smem_opt_in(reinterpret_cast<const void*>(k_descriptors_b<TX, TY>), smem, done_b)) != cudaSuccess) return e;
         k_descriptors_b<TX, TY><<<dim3(tiles, (unsigned)b.n), DESC_THREADS, smem, st>>>(b, t[0], t[1], t[2], prm.scale,

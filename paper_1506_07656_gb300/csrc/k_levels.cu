@@ -79,7 +79,10 @@ __device__ __forceinline__ void valid_all(const ValidArgs& a) {
     }
 }
 
-__global__ void __launch_bounds__(VALID_THREADS) k_valid_all(const __grid_constant__ ValidArgs a) { valid_all(a); }
+__global__ void __launch_bounds__(VALID_THREADS) k_valid_all(const __grid_constant__ ValidArgs a) {
+    dm_pdl_wait();
+    valid_all(a);
+}
 __global__ void __launch_bounds__(VALID_THREADS) k_valid_all_b(const __grid_constant__ ValidBatch B) {
     valid_all(B.a[blockIdx.y]);
 }
@@ -783,6 +786,7 @@ __global__ void __launch_bounds__(LV_THREADS, 4)
 k_level_rows(DmGeom g, int l, const float* __restrict__ prev, const unsigned char* __restrict__ vprev, int nbx, int nby,
              int seg_rows, float* __restrict__ out, unsigned char* __restrict__ amax, float lam,
              const int* __restrict__ proto_of, int n_maps) {
+    dm_pdl_wait();
     level_rows_body<COMP, LPP>(g, l, prev, vprev, nbx, nby, seg_rows, out, amax, lam, proto_of, n_maps, blockIdx.x);
 }
 
@@ -792,6 +796,7 @@ __global__ void k_level_top(DmGeom g, int l, const unsigned char* __restrict__ v
                             const unsigned char* __restrict__ vcur, const float* __restrict__ prev,
                             float* __restrict__ top, float lam, const int* __restrict__ proto_of, int n_maps) {
     const int p = blockIdx.y;
+    dm_pdl_wait();
     if (!vcur[p]) return;
     const int mw = g.dw[l], mh = g.dh[l];
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -858,10 +863,9 @@ cudaError_t launch_rows_lpp(const DmGeom& g, int l, const dm_pyramid& py, const 
     static std::atomic<unsigned long long> l1_done{0};
     const cudaError_t e = dm_prefer_l1(reinterpret_cast<const void*>(k_level_rows<COMP, LPP>), l1_done);
     if (e != cudaSuccess) return e;
-    k_level_rows<COMP, LPP><<<(unsigned)s.blocks, LV_THREADS, 0, st>>>(
-        g, l, py.pooled[l - 1], py.valid[l - 1], s.nbx, s.nby, s.seg_rows, const_cast<float*>(py.pooled[l]),
+    return dm_launch_pdl(
+        k_level_rows<COMP, LPP>, (unsigned)s.blocks, LV_THREADS, 0, st, g, l, py.pooled[l - 1], py.valid[l - 1], s.nbx, s.nby, s.seg_rows, const_cast<float*>(py.pooled[l]),
         const_cast<unsigned char*>(py.amax[l]), lam, l == 1 ? py.proto_of : nullptr, py.n0_maps);
-    return cudaGetLastError();
 }
 
 template <bool COMP>
@@ -974,7 +978,7 @@ cudaError_t dm_launch_levels(const DmGeom& g, const dm_pyramid& py, float lam, i
     const int B = 128;
     int n0 = g.npatch(0), np = g.npatch(1);
     const bool whole = valid_fits(g);
-    if (whole) k_valid_all<<<valid_blocks(max(n0, np)), VALID_THREADS, 0, st>>>(valid_args(py));
+    if (whole) dm_launch_pdl(k_valid_all, valid_blocks(max(n0, np)), VALID_THREADS, 0, st, valid_args(py));
     else k_fill_u8<<<(n0 + 255) / 256, 256, 0, st>>>(const_cast<unsigned char*>(py.valid[0]), n0, 1);
     for (int l = 1; l <= g.L; l++) {
         if (!whole) k_valid<<<(np + 255) / 256, 256, 0, st>>>(g, l, py.valid[l - 1], const_cast<unsigned char*>(py.valid[l]));
@@ -1021,8 +1025,8 @@ cudaError_t dm_launch_levels(const DmGeom& g, const dm_pyramid& py, float lam, i
             int n = g.dw[l] * g.dh[l];
             dim3 grid((n + B - 1) / B, np);
             auto kern = py.compensated ? k_level_top<true> : k_level_top<false>;
-            kern<<<grid, B, 0, st>>>(g, l, py.valid[l - 1], py.valid[l], py.pooled[l - 1], const_cast<float*>(py.top), lam,
-                                     l == 1 ? py.proto_of : nullptr, py.n0_maps);
+            dm_launch_pdl(kern, grid, B, 0, st, g, l, py.valid[l - 1], py.valid[l], py.pooled[l - 1], const_cast<float*>(py.top),
+                          lam, l == 1 ? py.proto_of : nullptr, py.n0_maps);
         }
     }
     dm_count_launches(1 + (whole ? 1 : 2) * g.L);
