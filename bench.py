@@ -786,12 +786,11 @@ def _measure_batch_uniform(dm, torch, dist, ctx, a, world, local, rank, W, H, np
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the
 # current kernels, from one ncu capture of one 1024x436 BF16 pair (one pass per
-# launch; profiles/ has the command): level 0 2.038 GB read + 16.235 GB written;
-# the level pass (k_level_sweep with 8-row tiles for levels 1-4, k_level_stream
-# for 5-7, k_level_top) 20.510 GB read + 5.122 GB written.  The FP32 level-0 kernel is
-# the capture at 512x224 scaled by the number of pooled outputs (x 15.1); FP8
-# has no capture of its current epilogue (None).
-TRAFFIC_1024x436 = {"level0_bf16": 18.27e9, "level0_fp8": None, "level0_fp32": 14.8e9, "levels": 25.63e9}
+# launch; profiles/ has the command): level 0 0.314 GB read + 15.538 GB written (FP8
+# 0.208 + 15.539); the level pass (k_level_rows for levels 1-7, k_level_top) 20.08 GB
+# read + 5.11 GB written.  The FP32 level-0 kernel is the capture at 512x224 scaled by
+# the number of pooled outputs (x 15.1).
+TRAFFIC_1024x436 = {"level0_bf16": 15.85e9, "level0_fp8": 15.75e9, "level0_fp32": 14.8e9, "levels": 25.19e9}
 
 
 def _prec_code(dm, name):
@@ -835,7 +834,7 @@ def _rooflines(r, prec, W, H, peaks, nsm):
     gbs = (rd + wr) / (lev_ms / 1e3) / 1e9
     lev = {"bound": "hbm", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
            "traffic": TRAFFIC_1024x436["levels"] if (W, H) == (1024, 436) else None,
-           "kernel": "k_level_sweep + k_level_stream (levels 1..L-1) + k_level_top (pyramid levels >= 1)",
+           "kernel": "k_level_rows / k_level_sweep (levels 1..L-1) + k_level_top (pyramid levels >= 1)",
            "peak_source": "hbm_gbs of measured" if "hbm_gbs" in peaks else "fallback 6.8 TB/s",
            "algorithmic_bytes_per_launch_set": rd + wr, "launch_ms": lev_ms}
     return corr, lev
