@@ -478,9 +478,9 @@ dm_status dm_set_batch_wave(dm_ctx* ctx, int pairs);
  * size's own).  chosen (may be NULL) receives {W, K}.  Synchronises with the host
  * (not capturable); the pairs' outputs hold the matches of the last run.
  * DM_ENOMEM if ws_bytes is below one lane_bytes.  Measured at 1024 x 436 (8
- * BF16 pairs, one graph): W = 1 on 2 lanes 61.6 pairs/s, waves of 2 on 2
- * lanes 60.1, W = 1 on 3 lanes 58.1, waves of 4 on one lane 57.9, W = 1 on
- * one lane 57.6 -- there one pair's kernels already fill the GPU and two
+ * BF16 pairs, one graph): W = 1 on 2 lanes 73.7 pairs/s, waves of 2 on 2
+ * lanes 73.3, W = 1 on 3 lanes 72.9, waves of 4 on one lane 70.1, W = 1 on
+ * one lane 68.3 -- there one pair's kernels already fill the GPU and two
  * lanes overlap one pair's latency-bound steps with another's level 0. */
 dm_status dm_autotune_batch(dm_ctx* ctx, int n, const dm_pair* pairs, void* d_ws, size_t ws_bytes, int* chosen,
                             void* stream);
