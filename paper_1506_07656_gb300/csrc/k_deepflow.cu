@@ -14,11 +14,11 @@
 //
 // The SOR sweeps are sequential in time (each half-sweep needs the other
 // colour's previous values), so the latency of a half-sweep and the launches,
-// not the arithmetic, bound the solver: the smaller levels (up to 4096 pixels) run
+// not the arithmetic, bound the solver: the smaller levels (up to 1024 pairs of pixels) run
 // entirely in one CTA; larger levels run 8 half-sweeps per launch, temporally blocked
 // (a tile plus an 8-pixel halo), which gives the same bits as 8 global half-sweeps.
-// In both a thread keeps the weights and increments of its pixels in registers and
-// reads only its neighbours' current values from shared memory.
+// In both a thread keeps the edge weights and increments of its pixels in registers and reads
+// its neighbours' current values and the constants of its own update from shared memory.
 #include <math.h>
 
 #include "dm_internal.cuh"
@@ -185,8 +185,10 @@ __global__ void k_df_prep2(const float* __restrict__ Im, int w, int h, float* __
 // dx(I1), Iyz = dy(I2w) - dy(I1); theta0 = 1 / (Ix^2 + Iy^2 + zeta^2),
 // thetax = 1 / (Ixx^2 + Ixy^2 + zeta^2), thetay = 1 / (Ixy^2 + Iyy^2 + zeta^2).
 __global__ void k_df_prep3(const float* __restrict__ I1, const float* __restrict__ I2w, const float* __restrict__ Ixa,
-                           const float* __restrict__ Iya, int w, int h, DfConst k, float* __restrict__ D) {
+                           const float* __restrict__ Iya, int w, int h, DfConst k, float* __restrict__ D,
+                           unsigned int* __restrict__ published) {
     const long long n = (long long)w * h;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *published = 0u;        // for the level's fixed-point steps (k_df_weights)
     for (long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x; o < n; o += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(o % w), y = (int)(o / w);
         const float Ix = Ixa[o], Iy = Iya[o];
@@ -329,7 +331,7 @@ struct SorPx {
 // corrections (Markstein: the remainder of an fma is exact, and with a correctly
 // rounded reciprocal the correction of a quotient that is off by less than an ulp
 // rounds correctly).  Outside the range where no remainder can underflow -- and
-// for the d that dm_sor_setup marks with lo = infinity -- the division itself.
+// for the d that sor_setup marks with lo = infinity -- the division itself.
 __device__ __forceinline__ float df_div(float a, float d, float y, float lo) {
     const float m = fabsf(a);
     if (!(m >= lo && m <= 1.0e24f)) return __fdiv_rn(a, d);
@@ -383,9 +385,20 @@ __device__ __forceinline__ void sor_update(SorPx& p, float2* mine, const float2*
     *mine = make_float2(__fadd_rn(p.du, p.u), __fadd_rn(p.dv, p.v));
 }
 
-__global__ void k_df_weights(DfLevel L, DfConst k) {
+// The systems and smoothness weights of a fixed-point step; every CTA publishes its share by a
+// release (its threads' writes are ordered before it by the barrier), so that whoever
+// acquires the count of all CTAs may read them, and what this kernel found written (u, v).
+__global__ void k_df_weights(DfLevel L, DfConst k, unsigned int* published) {
     for (long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x; o < L.n; o += (long long)gridDim.x * blockDim.x)
         df_weights_at(L, k, o);
+    __syncthreads();
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(published) : "memory");
+}
+
+__device__ __forceinline__ bool df_acquired(const unsigned int* published, unsigned int count) {
+    unsigned int c;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(published) : "memory");
+    return c == count;
 }
 
 // Temporally blocked red-black SOR: a CTA owns a TB_W x TB_H tile and stages
@@ -407,18 +420,18 @@ constexpr int TB_PLANE = TB_PAIRS + 2 * TB_PW;                   // with guards
 constexpr size_t TB_SMEM = (size_t)(4 * TB_PLANE + 2 * SOR_INV * TB_PAIRS) * sizeof(float);
 static_assert(TB_S % 2 == 0 && TB_W % 2 == 0, "a launch starts with colour 0 and the staged region at an even column");
 
-// Launches of one fixed-point step follow one another with programmatic dependence:
-// what a launch reads that the one before it does not write (u, v, ps, A) is staged
-// before it waits for that one (`early`; the first launch waits first, since the
-// kernel before it writes them), and only its increments after.  Every launch lets
-// its successor start after its own wait, so a launch that starts early knows the
-// kernel before its predecessor to have ended.
-__global__ void __launch_bounds__(TB_THREADS, 2) k_df_sor_tb(DfLevel L, DfConst k, int S, int early, float* __restrict__ out_du,
+// Every launch depends programmatically on the one before it (dm_launch_pdl): its CTAs become
+// resident while that one's last ones run.  What it reads that its predecessor does not
+// write (u, v, ps, A) it stages meanwhile, and only its increments after the wait.  The wait
+// covers the predecessor alone, so the early reads are ordered by the count that
+// k_df_weights publishes: a thread that acquires `count` (the CTAs of all weights launches
+// of the level so far) reads what that kernel wrote or found written; any other value --
+// and count = 0, the first launch of a step, whose predecessor is the weights kernel
+// -- and it waits first.
+// (Everything staged after the wait: a 1024x436 pair 22.3 ms instead of 20.4.)
+__global__ void __launch_bounds__(TB_THREADS, 2) k_df_sor_tb(DfLevel L, DfConst k, int S, const unsigned int* published,
+                                                             unsigned int count, float* __restrict__ out_du,
                                                              float* __restrict__ out_dv) {
-    if (!early) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    }
     extern __shared__ __align__(16) float sm[];
     // per colour: the sums, the constants of this thread's pixel
     float2* cur[2] = {reinterpret_cast<float2*>(sm) + TB_PW + threadIdx.x,
@@ -439,6 +452,8 @@ __global__ void __launch_bounds__(TB_THREADS, 2) k_df_sor_tb(DfLevel L, DfConst 
     int act[2];                                          // half-sweeps in which the pixel is updated: j < act
     float ps[2], A[2][5];
     bool in[2];
+    const bool early = count != 0u && df_acquired(published, count);
+    if (!early) dm_pdl_wait();
 #pragma unroll
     for (int c = 0; c < 2; c++) {
         const int x = 2 * i + (c ^ flip);
@@ -470,15 +485,12 @@ __global__ void __launch_bounds__(TB_THREADS, 2) k_df_sor_tb(DfLevel L, DfConst 
         ok = ok && (good || act[c] <= 0);
     }
     __syncthreads();                                     // ps read
-    if (early) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    }
+    if (early) dm_pdl_wait();
 #pragma unroll
     for (int c = 0; c < 2; c++) {
         const long long o = in[c] ? (long long)gy * L.w + (lx0 + 2 * i + (c ^ flip)) : 0;
-        px[c].du = __ldcg(L.du + o);                     // (written by the launch before)
-        px[c].dv = __ldcg(L.dv + o);
+        px[c].du = L.du[o];
+        px[c].dv = L.dv[o];
         cur[c][0] = make_float2(__fadd_rn(px[c].du, px[c].u), __fadd_rn(px[c].dv, px[c].v));
         if (threadIdx.x < TB_PW) cur[c][-TB_PW] = cur[c][TB_PAIRS] = make_float2(0.0f, 0.0f);
     }
@@ -598,24 +610,6 @@ __global__ void __launch_bounds__(DF_SMALL_THREADS) k_df_level_small(DfLevel L, 
 // ---------------------------------------------------------------------------
 namespace {
 constexpr double kPi = 3.14159265358979323846;
-// One blocked SOR launch, with programmatic dependence on the kernel before it.
-cudaError_t launch_sor_tb(unsigned tiles, const DfLevel& L, const DfConst& k, int S, bool early, float* out_du, float* out_dv,
-                          cudaStream_t st) {
-    cudaLaunchAttribute attr;
-    memset(&attr, 0, sizeof(attr));
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(tiles);
-    cfg.blockDim = dim3(TB_THREADS);
-    cfg.dynamicSmemBytes = TB_SMEM;
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_df_sor_tb, L, k, S, early ? 1 : 0, out_du, out_dv);
-}
-
 inline unsigned df_blocks(long long n) {
     const long long b = (n + 255) / 256;
     return (unsigned)(b < 4096 ? (b > 0 ? b : 1) : 4096);
@@ -730,10 +724,13 @@ cudaError_t dm_launch_deepflow(const DmFlowPlan& q, const DmTaps& taps, const fl
         }
         k_df_match_fields<<<df_blocks(n), 256, 0, st>>>(owner, m, F(q.phi), (int)n, q.beta_k[l], q.sk[l], F(q.mc), F(q.mu),
                                                          F(q.mv));
-        // linearisation around the current flow
+        // linearisation around the current flow (Im is free after the second step: its first word counts
+        // the CTAs of the weights launches)
+        unsigned int* published = reinterpret_cast<unsigned int*>(F(q.Im));
         k_df_prep1<<<df_blocks(n), 256, 0, st>>>(F(q.P1[l]), F(q.P2[l]), cu, cv, w, h, k, F(q.alpha), F(q.I2w), F(q.Im));
         k_df_prep2<<<df_blocks(n), 256, 0, st>>>(F(q.Im), w, h, F(q.Ix), F(q.Iy));
-        k_df_prep3<<<df_blocks(n), 256, 0, st>>>(F(q.P1[l]), F(q.I2w), F(q.Ix), F(q.Iy), w, h, k, F(q.D));
+        k_df_prep3<<<df_blocks(n), 256, 0, st>>>(F(q.P1[l]), F(q.I2w), F(q.Ix), F(q.Iy), w, h, k, F(q.D),
+                                                   published);
         launches += 4;
         if ((e = cudaMemsetAsync(F(q.du), 0, n * 4, st)) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(F(q.dv), 0, n * 4, st)) != cudaSuccess) return e;
@@ -751,11 +748,14 @@ cudaError_t dm_launch_deepflow(const DmFlowPlan& q, const DmTaps& taps, const fl
             float* alt_u = F(q.du2);
             float* alt_v = F(q.dv2);
             for (int it = 0; it < q.n_fixed; it++) {
-                k_df_weights<<<df_blocks(n), 256, 0, st>>>(L, k);
+                k_df_weights<<<df_blocks(n), 256, 0, st>>>(L, k, published);
                 launches++;
                 for (int j = 0; j < 2 * q.n_sor; j += TB_S) {
                     const int S = 2 * q.n_sor - j < TB_S ? 2 * q.n_sor - j : TB_S;
-                    if ((e = launch_sor_tb(tiles, L, k, S, j > 0, alt_u, alt_v, st)) != cudaSuccess) return e;
+                    const unsigned int count = j > 0 ? df_blocks(n) * (unsigned int)(it + 1) : 0u;
+                    if ((e = dm_launch_pdl(k_df_sor_tb, tiles, TB_THREADS, TB_SMEM, st, L, k, S, published, count, alt_u, alt_v)) !=
+                        cudaSuccess)
+                        return e;
                     launches++;
                     float* t = L.du; L.du = alt_u; alt_u = t;
                     t = L.dv; L.dv = alt_v; alt_v = t;
