@@ -1162,8 +1162,9 @@ cudaError_t dm_launch_levels_batch(const dm_pyramid* const* pys, int n, float la
                     const int kidf = (((2 * TH + 1) * KW + 31) / 32) * 32;     // LevelTile<TH>::KIDF
                     const size_t smem = (size_t)(NR * 2 * kidf + (2 * TH + 1) * AWP) * sizeof(float) + 128;
                     const int nt = TH == 16 ? level_threads<16>() : (TH == 8 ? level_threads<8>() : level_threads<4>());
-                    static std::atomic<unsigned long long> done[6];
-                    cudaError_t ea = dm_smem_opt_in(reinterpret_cast<const void*>(kern), (int)smem, done[shape - 1]);
+                    // (per kernel: this lambda has one instance, the kernels being of one type)
+                    static std::atomic<unsigned long long> done[6][2];
+                    cudaError_t ea = dm_smem_opt_in(reinterpret_cast<const void*>(kern), (int)smem, done[shape - 1][comp]);
                     if (ea != cudaSuccess) return ea;
                     kern<<<(unsigned)blocks, nt, smem, st>>>(B, l, lam);
                     return cudaSuccess;
