@@ -364,8 +364,10 @@ __device__ __forceinline__ bool sor_setup(SorPx& p, float* inv, int stride, floa
 // The other colour's neighbours of a pixel of pair e (planes of `pw` pairs per row): the
 // pixel of colour c lies at column 2 i + off of its row, its left and right
 // neighbours in pairs e - 1 + off and e + off, the upper and lower ones in e -+ pw.
-// (A neighbour that does not exist has weight 0, so any finite value serves: the
-// planes have `pw` guard elements before and after.)
+// A neighbour that does not exist has weight 0 and its element holds zeros: the planes have
+// guard elements before and after, and where a row could run into the next one (its end is
+// its successor's left neighbour) an element of padding.  (Weight 0 times whatever lies
+// there would carry a NaN or an infinity from one border to the other.)
 __device__ __forceinline__ void sor_update(SorPx& p, float2* mine, const float2* other, int off, int pw, const float* inv,
                                            int stride, float lo, const DfConst& k) {
     const float2 l = other[off - 1], r = other[off], t = other[-pw], b = other[pw];
@@ -491,7 +493,10 @@ __global__ void __launch_bounds__(TB_THREADS, 2) k_df_sor_tb(DfLevel L, DfConst 
         const long long o = in[c] ? (long long)gy * L.w + (lx0 + 2 * i + (c ^ flip)) : 0;
         px[c].du = L.du[o];
         px[c].dv = L.dv[o];
-        cur[c][0] = make_float2(__fadd_rn(px[c].du, px[c].u), __fadd_rn(px[c].dv, px[c].v));
+        // (zeros past the image's right and lower border; a staged region that has none to spare
+        // there ends 8 columns or rows past its tile, and what its last ones read does not
+        // reach the tile in 8 half-sweeps)
+        cur[c][0] = in[c] ? make_float2(__fadd_rn(px[c].du, px[c].u), __fadd_rn(px[c].dv, px[c].v)) : make_float2(0.0f, 0.0f);
         if (threadIdx.x < TB_PW) cur[c][-TB_PW] = cur[c][TB_PAIRS] = make_float2(0.0f, 0.0f);
     }
     const float lo = ok ? 1.0e-24f : INFINITY;
@@ -528,16 +533,18 @@ constexpr int DF_SMALL_THREADS = 1024;
 // Pairs of a level solved by one CTA (a row of w pixels holds (w + 1) / 2): with two
 // pairs per thread, up to 2048, a 1024x436 pair took 0.4 ms longer (spilled registers).
 constexpr int DF_SMALL_PAIRS = DF_SMALL_THREADS;
-constexpr size_t DF_SMALL_SMEM = (size_t)(DF_SMALL_PAIRS * 2 * (2 + SOR_INV + 1) + 8 * DF_SMALL_PAIRS) * sizeof(float);   // sums, constants, psi_s, guards
+// sums (two planes of h + 2 rows of pw + 1 elements, the guards and the padding among them: at most
+// 3 pairs + 3 for pw h <= pairs), constants, psi_s
+constexpr size_t DF_SMALL_SMEM = (size_t)(4 * (3 * DF_SMALL_PAIRS + 3) + 2 * (SOR_INV + 1) * DF_SMALL_PAIRS) * sizeof(float);
 
 __global__ void __launch_bounds__(DF_SMALL_THREADS) k_df_level_small(DfLevel L, DfConst k, int n_fixed, int n_sor) {
     extern __shared__ __align__(16) float sm[];
-    const int w = L.w, h = L.h, pw = (w + 1) / 2, np = pw * h, plane = np + 2 * pw;
+    const int w = L.w, h = L.h, pw = (w + 1) / 2, np = pw * h, row = pw + 1, plane = row * (h + 2);
     const long long n = L.n;
-    float2* cur[2] = {reinterpret_cast<float2*>(sm) + pw, reinterpret_cast<float2*>(sm) + plane + pw};
+    float2* cur[2] = {reinterpret_cast<float2*>(sm) + row, reinterpret_cast<float2*>(sm) + plane + row};
     float* inv[2] = {sm + 4 * plane, sm + 4 * plane + SOR_INV * np};
     float* sps[2] = {sm + 4 * plane + 2 * SOR_INV * np, sm + 4 * plane + (2 * SOR_INV + 1) * np};      // psi_s per colour
-    const int e = threadIdx.x, y = e / pw, i = e - y * pw, flip = y & 1;
+    const int e = threadIdx.x, y = e / pw, i = e - y * pw, flip = y & 1, at = y * row + i;      // the pair, its sums
     SorPx px[2];                                         // per colour, at column 2 i + (c ^ flip)
     bool in[2];
 #pragma unroll
@@ -550,8 +557,9 @@ __global__ void __launch_bounds__(DF_SMALL_THREADS) k_df_level_small(DfLevel L, 
             p.u = L.u[(long long)y * w + x];
             p.v = L.v[(long long)y * w + x];
         }
-        if (e < np) cur[c][e] = make_float2(p.u, p.v);   // du = dv = 0
-        if (e < pw) cur[c][e - pw] = cur[c][np + e] = make_float2(0.0f, 0.0f);
+        if (e < np) cur[c][at] = make_float2(p.u, p.v);  // du = dv = 0
+        if (e < np && i == pw - 1) cur[c][at + 1] = make_float2(0.0f, 0.0f);
+        for (int g = e; g < row; g += blockDim.x) cur[c][g - row] = cur[c][row * h + g] = make_float2(0.0f, 0.0f);
     }
     __syncthreads();
     for (int it = 0; it < n_fixed; it++) {
@@ -564,7 +572,7 @@ __global__ void __launch_bounds__(DF_SMALL_THREADS) k_df_level_small(DfLevel L, 
             const SorPx& p = px[c];
             const int x = 2 * i + (c ^ flip);
             const long long o = (long long)y * w + x;
-            const float2 r = cur[c ^ 1][e + (c ^ flip)], b = cur[c ^ 1][e + pw];
+            const float2 r = cur[c ^ 1][at + (c ^ flip)], b = cur[c ^ 1][at + row];
             float d[11];
             df_load_d(L.D, n, o, d);
             a[c] = df_weights_vals(p.u, p.du, p.v, p.dv, x + 1 < w, r.x, r.y, y + 1 < h, b.x, b.y, d, L.alpha[o], L.mc[o],
@@ -586,9 +594,9 @@ __global__ void __launch_bounds__(DF_SMALL_THREADS) k_df_level_small(DfLevel L, 
         }
         const float lo = ok ? 1.0e-24f : INFINITY;
         for (int s = 0; s < n_sor; s++) {
-            if (in[0]) sor_update(px[0], cur[0] + e, cur[1] + e, flip, pw, inv[0] + e, np, lo, k);
+            if (in[0]) sor_update(px[0], cur[0] + at, cur[1] + at, flip, row, inv[0] + e, np, lo, k);
             __syncthreads();
-            if (in[1]) sor_update(px[1], cur[1] + e, cur[0] + e, flip ^ 1, pw, inv[1] + e, np, lo, k);
+            if (in[1]) sor_update(px[1], cur[1] + at, cur[0] + at, flip ^ 1, row, inv[1] + e, np, lo, k);
             __syncthreads();
         }
     }
