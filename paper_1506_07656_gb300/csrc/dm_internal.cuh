@@ -634,6 +634,8 @@ cudaError_t dm_launch_kmeans(const DmGeom& g, const float* d1, int D, int iters,
                              int* assign, char* ws, cudaStream_t st);
 size_t dm_corr0_tc_a_bytes(const DmGeom& g, int precision);
 cudaError_t dm_launch_levels(const DmGeom& g, const dm_pyramid& p, float lam, int* status, cudaStream_t st);
+// Whether the tiled kernel takes level l (1 .. L-1) under these launch shapes.
+bool dm_level_tiled(const DmGeom& g, int l, const DmTune& tune);
 // The same for the n <= DM_BATCH_MAX pyramids of a wave (same precision and
 // child-sum mode, level 0 computed): one launch per kernel and level for all.
 cudaError_t dm_launch_levels_batch(const dm_pyramid* const* pys, int n, float lam, int* const* status, cudaStream_t st);

@@ -877,19 +877,27 @@ cudaError_t launch_rows(const DmGeom& g, int l, const dm_pyramid& py, const LvSh
     return launch_rows_lpp<COMP, 4>(g, l, py, s, lam, st);
 }
 
-// Which kernel takes level l: the row-streaming one where the tuned shape asks for it
-// (level_th = 0); for maps of at most 16 columns and for small images, where the tiled
-// kernel's per-patch pipeline is latency-bound; and for wider maps whose rows fill its
-// 64-column strips (or its one 32-column strip) to 88 %: it moves less through L1
-// and L2 than the tiled kernel, which has no such granularity.  A fault-injection run
-// takes the tiled kernel, which holds the bounded waits.  Measured (ncu, us, tiled /
-// row-streaming; columns of the stored map in front): 1024x436 256 5362 / 4487, 128
-// 1362 / 1137, 64 395 / 309, 32 117 / 113, 1242x375 311 (97 % filled) 6043 / 5484, 512x224
-// 128 370 / 311, 256x256 64 132 / 113; 640x480 160 (83 %) 2497 / 2806, 80 807 / 909, 20 80 / 115,
-// 1242x375 156 (81 %) 1535 / 1790; 130x70 33 41 / 29.
+// Which kernel takes level l.  The row-streaming one where the tuned shape asks for it
+// (level_th = 0) and for maps of at most 16 columns; for maps of up to 64 columns, where
+// they fill its strips (one of 64 or of 32) to 88 % or the image is small (the tiled
+// kernel's per-patch pipeline is then latency-bound); for wider maps where they fill strips of 64 to
+// 88 % and the patches are enough to hide its loads: it moves less through L1 and L2 than
+// the tiled kernel, which has no such granularity.  A fault-injection run takes the
+// tiled kernel, which holds the bounded waits.
+//   Measured (us, tiled / row-streaming; columns of the stored map in front): 1024x436 256
+// 5362 / 4487, 128 1362 / 1137, 64 395 / 309, 32 117 / 113, 1242x375 311 (97 % filled) 6043 /
+// 5484, 512x224 128 370 / 311, 256x256 64 132 / 113; 640x480 160 (in strips of 32) 2497 / 2806,
+// 80 807 / 909, 20 80 / 115, 1242x375 156 1535 / 1790; 130x70 33 41 / 29.
+//   Image 1 of few patches (what the tiled kernel adds to a call of dm_correlate_pyramid): maps
+// of 40 columns, patches in front: 144 +9, 576 +10, 1024 +11, 1936 +13; 80 columns: 144 -15,
+// 576 -24, 1024 -29, 1936 -21; 160: -42, -38, -41, -48; 256 (filled): 144 -19, 576 +11, 1024
+// +28; 311 (filled): 144 -36, 400 -26, 576 -14, 1024 +1, 1936 +28.
 bool level_streams(const DmGeom& g, int l, const DmTune& tune, const LvShape& s) {
-    const int ow = g.dw[l + 1];
-    return tune.level_th == 0 || ow <= 16 || g.npatch(l) <= 2048 || (s.fill >= 0.88 && (s.lpp == 32 || ow <= 32));
+    const int ow = g.dw[l + 1], np = g.npatch(l);
+    if (tune.level_th == 0 || ow <= 16) return true;
+    const bool filled = s.fill >= 0.88;
+    if (ow <= 64) return np <= 2048 || (filled && (s.lpp == 32 || ow <= 32));
+    return filled && s.lpp == 32 && np >= 512;
 }
 
 // ---------------------------------------------------------------------------
@@ -973,6 +981,10 @@ __global__ void k_level_top_b(const __grid_constant__ LvBatch B, int l, float la
 }
 
 }  // namespace
+
+bool dm_level_tiled(const DmGeom& g, int l, const DmTune& tune) {
+    return l >= 1 && l < g.L && !level_streams(g, l, tune, level_shape(g, l));
+}
 
 cudaError_t dm_launch_levels(const DmGeom& g, const dm_pyramid& py, float lam, int* status, cudaStream_t st) {
     const int B = 128;
