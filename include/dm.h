@@ -495,13 +495,15 @@ dm_status dm_autotune_batch(dm_ctx* ctx, int n, const dm_pair* pairs, void* d_ws
  *              or 8 chunks; unused by DM_FP32);
  *   chosen[1]  level kernel: pooled rows per CTA tile of the tiled kernel (16,
  *              8 or 4, on 8, 4 or 2 warps), or 0 for the row-streaming kernel
- *              (registers only, strips of 64 columns) at every level; levels
- *              whose stored maps are at most 16 columns wide or fill its strips,
- *              and small images, always take the latter;
+ *              (strips of 64 columns in registers) at every level.  With a tile,
+ *              levels whose stored maps are at most 16 columns wide or fill
+ *              the strips still take the row-streaming kernel, and with 8 rows
+ *              and a ring of 2 (the default) so do the maps of up to 64 columns
+ *              of images of up to 2048 patches;
  *   chosen[2]  CTAs per SM of the backtracking expansion kernels (2..32);
  *   chosen[3]  child-window columns in the level kernel's ring (3 or 2).
- * Every candidate computes identical results; only the time differs.  Each
- * candidate runs three times (after one untimed run of the default), timed
+ * Every candidate computes identical results; only the time differs.  A tile that
+ * no level would take is not tried.  Each candidate runs three times (after one untimed run of the default), timed
  * with CUDA events, best of three; a candidate replaces the current choice
  * only when it is at least 3% faster.  Later
  * dm_correlate_pyramid / dm_match / dm_match_batch calls on pairs of these

@@ -1311,7 +1311,15 @@ dm_status dm_autotune(dm_ctx* ctx, const float* d_img1, int W1, int H1, const fl
     cur = timed(levels);
     // rows per tile x ring (the default first, timed above); 0 = row-streaming kernel
     const int lshapes[6][2] = {{16, 2}, {16, 3}, {8, 3}, {4, 2}, {4, 3}, {0, 2}};
+    auto tiled = [&](int th, int ring) {             // some level takes the tiled kernel
+        const DmTune t{best.m_chunk, th, best.bt_mult, ring};
+        for (int l = 1; l < g.L; l++)
+            if (dm_level_tiled(g, l, t)) return true;
+        return false;
+    };
+    const bool default_tiled = tiled(best.level_th, best.level_ring);
     for (const auto& sh : lshapes) {
+        if (!default_tiled && !tiled(sh[0], sh[1])) continue;      // the same kernels as the default's
         py.tune.level_th = sh[0];
         py.tune.level_ring = sh[1];
         if (pick(timed(levels), cur)) { best.level_th = sh[0]; best.level_ring = sh[1]; }

@@ -880,7 +880,8 @@ cudaError_t launch_rows(const DmGeom& g, int l, const dm_pyramid& py, const LvSh
 // Which kernel takes level l.  The row-streaming one where the tuned shape asks for it
 // (level_th = 0) and for maps of at most 16 columns; for maps of up to 64 columns, where
 // they fill its strips (one of 64 or of 32) to 88 % or the image is small (the tiled
-// kernel's per-patch pipeline is then latency-bound); for wider maps where they fill strips of 64 to
+// kernel's per-patch pipeline is then latency-bound; not where another tile than the default
+// was set, which is a request for it); for wider maps where they fill strips of 64 to
 // 88 % and the patches are enough to hide its loads: it moves less through L1 and L2 than
 // the tiled kernel, which has no such granularity.  A fault-injection run takes the
 // tiled kernel, which holds the bounded waits.
@@ -895,8 +896,8 @@ cudaError_t launch_rows(const DmGeom& g, int l, const dm_pyramid& py, const LvSh
 bool level_streams(const DmGeom& g, int l, const DmTune& tune, const LvShape& s) {
     const int ow = g.dw[l + 1], np = g.npatch(l);
     if (tune.level_th == 0 || ow <= 16) return true;
-    const bool filled = s.fill >= 0.88;
-    if (ow <= 64) return np <= 2048 || (filled && (s.lpp == 32 || ow <= 32));
+    const bool filled = s.fill >= 0.88, default_tile = tune.level_th == 8 && tune.level_ring == 2;
+    if (ow <= 64) return (np <= 2048 && default_tile) || (filled && (s.lpp == 32 || ow <= 32));
     return filled && s.lpp == 32 && np >= 512;
 }
 

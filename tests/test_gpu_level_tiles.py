@@ -52,3 +52,69 @@ def test_waves_of_both_child_sums(dm_mod, rows, ring):
                 np.testing.assert_array_equal(out[:int(cnt.item())].cpu().numpy(), want)
         finally:
             ctx.close()
+
+
+def _check_levels(dm, ws, h, pyr):
+    for l in range(1, pyr.geom.L + 1):
+        vals, codes, valid = dm.read_level(ws, dm.dm_pyramid_level(h, l))
+        np.testing.assert_array_equal(valid, pyr.valid[l])
+        keep = valid.astype(bool)
+        np.testing.assert_array_equal(vals[keep], (pyr.pooled[l] if l < pyr.geom.L else pyr.top)[keep], err_msg=f"level {l}")
+        if l < pyr.geom.L:
+            np.testing.assert_array_equal(codes[keep], pyr.argmax[l][keep], err_msg=f"level {l} codes")
+
+
+@pytest.mark.parametrize("compensated", [True, False])
+@pytest.mark.parametrize("size", [(W1, H1, W2, H2), (130, 70, 133, 71)])
+def test_every_tile_bit_exact(dm_mod, oracle_mod, size, compensated):
+    """Every tile and ring, the default's too, against the FP32 oracle at every level >= 1 (tests/test_level_routes.py
+    says which levels of these sizes are tiled: two, with the default tile only at the first size)."""
+    import torch
+    dm = dm_mod
+    w1, h1, w2, h2 = size
+    rng = np.random.default_rng(7)
+    d1 = oracle_mod.descriptors(synth.value_noise(w1, h1, rng).astype(np.float32), "f32")
+    d2 = oracle_mod.descriptors(synth.value_noise(w2, h2, rng).astype(np.float32), "f32")
+    pyr = oracle_mod.pyramid(d1, d2, "f32", compensated=compensated)
+    t1, t2 = torch.from_numpy(d1).cuda(), torch.from_numpy(d2).cuda()
+    ctx = dm.Context(dm.DM_FP32, compensated=int(compensated))
+    try:
+        ws = torch.empty(dm.dm_workspace_bytes(ctx.ctx, *size)["pyramid"], dtype=torch.uint8, device="cuda")
+        for rows in (16, 8, 4):
+            for ring in (2, 3):
+                ws.fill_(0xA5)
+                dm.dm_set_tuned_config(ctx.ctx, *size, {"m_chunk": 1, "level_tile_rows": rows, "bt_ctas_per_sm": 8,
+                                                        "level_ring": ring})
+                h = dm.dm_correlate_pyramid(ctx.ctx, t1, t2, ws)
+                try:
+                    _check_levels(dm, ws, h, pyr)
+                finally:
+                    dm.dm_pyramid_free(h)
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("compensated", [True, False])
+def test_approximate_form_bit_exact(dm_mod, oracle_mod, compensated):
+    """The tiled instances that read level 0 through the prototype index (level 1), against the FP32 oracle's chain on
+    the patches replaced by their prototypes."""
+    import torch
+    dm = dm_mod
+    a, b = _images(3)
+    rng = np.random.default_rng(4)
+    vecs = oracle_mod.patch_vectors(oracle_mod.descriptors(a, "f32"))
+    protos = np.ascontiguousarray(vecs[rng.choice(len(vecs), 37, replace=False)])
+    assign = rng.integers(0, 37, len(vecs)).astype(np.int32)
+    _, pyr, _ = oracle_mod.approx_match(a, b, protos, assign, "f32", compensated=compensated)
+    d2 = torch.from_numpy(oracle_mod.descriptors(b, "f32")).cuda()
+    tp, ta = torch.from_numpy(protos).cuda(), torch.from_numpy(assign).cuda()
+    ctx = dm.Context(dm.DM_FP32, compensated=int(compensated))
+    try:
+        ws = torch.full((dm.dm_workspace_bytes(ctx.ctx, W1, H1, W2, H2)["pyramid"],), 0xA5, dtype=torch.uint8, device="cuda")
+        h = dm.dm_correlate_pyramid_approx(ctx.ctx, tp, ta, W1, H1, d2, ws)
+        try:
+            _check_levels(dm, ws, h, pyr)
+        finally:
+            dm.dm_pyramid_free(h)
+    finally:
+        ctx.close()

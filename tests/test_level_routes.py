@@ -1,10 +1,10 @@
-"""Which kernel takes a level (tiled or row-streaming), by the library's own rule: small images and filled maps stream, and
-a small image 1 does not pull the wide maps of a larger image 2 along."""
+"""Which kernel takes a level (tiled or row-streaming), by the library's own rule: small images and filled maps stream, a
+tile that was set is taken, and a small image 1 does not pull the wide maps of a larger image 2 along."""
 import ctypes as C
 
 import pytest
 
-SMALL = (8, 2)                          # (rows, ring): the default tile
+SMALL, SET = (8, 2), (8, 3)             # (rows, ring): the default tile, another one
 
 
 @pytest.fixture(scope="module")
@@ -26,9 +26,10 @@ def tiled():
 
 
 @pytest.mark.parametrize("pair,tile,want", [
-    # maps of 33 and 17 columns (25, then 13), small images: streaming
-    ((130, 70, 130, 70), SMALL, []),
-    ((97, 61, 97, 61), SMALL, []),
+    # maps of 33 and 17 columns (25, then 13), small images: streaming, unless a tile is set
+    ((130, 70, 133, 71), SET, [1, 2]), ((300, 124, 160, 96), (16, 3), [1, 2]),
+    ((130, 70, 130, 70), SMALL, []), ((130, 70, 130, 70), SET, [1, 2]), ((130, 70, 130, 70), (16, 2), [1, 2]),
+    ((97, 61, 97, 61), SMALL, []), ((97, 61, 97, 61), (4, 3), [1]),
     ((64, 48, 64, 48), SMALL, []), ((130, 70, 130, 70), (0, 2), []),
     # image 1 of 144 and 1936 patches, maps of 160, 80, 40 and 20 columns
     ((48, 48, 640, 480), SMALL, [1, 2]), ((176, 176, 640, 480), SMALL, [1, 2]), ((48, 48, 320, 240), SMALL, [1]),
