@@ -17,6 +17,15 @@
 // staged into a second buffer meanwhile (asynchronous 4-byte copies, zero-filled
 // outside the images: a pixel's nine floats allow no wider ones).
 //
+// The bands of a patch group lie side by side in one row of tiles, so that a map's last
+// columns and the next band's first ones share a tile: one empty lane after each band, whose
+// pixels are zeros, is border enough for both (a position needs two pixels to the left and one
+// to the right).  Where the columns fill whole tiles, or on small inputs where that makes no
+// SM's tiles fewer, a band takes whole tiles instead.  With whole tiles for every width up to
+// 62 % of the lanes were idle.  dm_correlate_pyramid, whole tiles / so / tiles of 15 columns with
+// one lane per column: 256x256 against 24x200 (map of 12 columns) 521 / 353 / 445 us, 200x200 1091
+// / 903 / 1058, 512x224 5701 / 5714 / 7085.
+//
 // Work of a CTA: an equal range of the tiles in the order (patch group, band, column),
 // about one CTA per SM and at most RANGE tiles each, so that the last wave is a full
 // one (13.5 waves of whole bands took 14).  Small inputs have fewer tiles than SMs: they
@@ -85,6 +94,9 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return r;
 }
 
+// Tiles of a patch group's row of bands, `bl` lanes each.
+__host__ __device__ inline int band_tiles(int bands, int bl) { return (bands * bl + PWT - 1) / PWT; }
+
 // The maximum of a column over the three rows of a pooled row, and 3 x the first row
 // reaching it, shifted by sh.
 __device__ __forceinline__ float col_max(float v0, float v1, float v2, int sh, uint32_t& y3) {
@@ -97,38 +109,48 @@ template <int PH, int NP>
 __global__ void __launch_bounds__(256, Band<PH, NP>::CTAS_SM)
 k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2, float lam,
             float* __restrict__ pooled0, unsigned char* __restrict__ amax0, const float* __restrict__ amat, int n0,
-            long long units) {
+            long long units, int bl) {
     using B = Band<PH, NP>;
     constexpr int CROWS = B::CROWS, HROWS = B::HROWS, PLANE = B::PLANE, COPY = B::COPY, PATCHES = B::PATCHES;
     extern __shared__ __align__(16) float sm[];
-    // a buffer: even [9][HROWS][HPITCH], column j = pixel 64 t - 2 + j, and odd, the same
-    // shifted, column j = pixel 64 t - 1 + j
+    // a buffer: even [9][HROWS][HPITCH], the pixels of lane j at columns 2 j + 2 and 2 j + 3, two more before
+    // and one after them, and odd, the same shifted by one
     float2* a_s = reinterpret_cast<float2*>(sm + B::BUFS * 2 * COPY);    // [(dx*9+c)*4+dy][patch], value twice
     float* left_s = sm + B::BUFS * 2 * COPY + 144 * PATCHES * 2;         // [warp][patch][LEFT]
-    float* edge = left_s + WARPS * NP * LEFT;                            // [9][HROWS]: pixel 64 t - 3 of the first tile
+    float* edge = left_s + WARPS * NP * LEFT;                            // [9][HROWS]: the pixel before those of the first tile
 
     const int W2 = g.W2, H2 = g.H2, mw = g.dw[1], mh = g.dh[1], pitch = g.pitch(1);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int tiles = (mw + PWT - 1) / PWT, bands = (mh + PH - 1) / PH;
+    const int bands = (mh + PH - 1) / PH, tiles = band_tiles(bands, bl);
     const long long u0 = units * blockIdx.x / gridDim.x;
     int todo = (int)(units * (blockIdx.x + 1) / gridDim.x - u0);
-    int t = (int)(u0 % tiles), ry0 = (int)(u0 / tiles % bands) * PH, p_base = (int)(u0 / tiles / bands) * PATCHES;
-    bool load = true, edged = t > 0;                     // stage the patch vectors, form the column before the tile
+    int t = (int)(u0 % tiles), p_base = (int)(u0 / tiles) * PATCHES;
+    int b0 = PWT * t / bl, c0 = PWT * t - b0 * bl;       // lane 0's band and its pooled column
+    // stage the patch vectors; form the column before the first tile, where that begins inside a band
+    bool load = true, edged = c0 > 0 && c0 < mw;
     const DmPow pr = dm_pow_setup(lam);
     dm_pdl_wait();
 
-    // image-2 descriptors of pixels [64 t - 2, 64 t + 65) x [2 ry0 - 3, 2 ry0 - 3 + HROWS), zero
-    // outside I': a row of them is 603 consecutive floats
-    auto stage = [&](int t, int ry0, float* even) {
-        const int y0 = 2 * ry0 - 3;
-        const bool full = t > 0 && 2 * PWT * t + 2 * PWT + 1 <= W2 && y0 >= 0 && y0 + HROWS <= H2;
+    // band and pooled column of a lane past the end of band b
+    auto wrap = [&](int& b, int& c) {
+        while (c >= bl) {
+            c -= bl;
+            b++;
+        }
+    };
+
+    // image-2 descriptors of a tile, zero outside I': the pixels of lane j and one row of them per
+    // staged row of its band (a band's first row is 3 above its C0 rows' centres)
+    auto stage = [&](int b0, int c0, float* even) {
+        const int y00 = 2 * PH * b0 - 3;
+        // a tile inside a band and inside I': a row of it is 603 consecutive floats
+        const bool full = c0 > 0 && 2 * (c0 + PWT) + 1 <= W2 && y00 >= 0 && y00 + HROWS <= H2;
         for (int q = tid; q < HCOLS * 9; q += 256) {
             const int col = q / 9, c = q - 9 * col;
-            const int x9 = (2 * PWT * t - 2) * 9 + q;
-            const float* src = d2 + (long long)y0 * W2 * 9 + x9;
             float* e = even + c * PLANE + col;
             float* o = even + COPY + c * PLANE + col - 1;
             if (full && col >= 1 && col < HPITCH) {
+                const float* src = d2 + (long long)y00 * W2 * 9 + (2 * c0 - 2) * 9 + q;
 #pragma unroll
                 for (int r = 0; r < HROWS; r++) {
                     cp_async4(e + r * HPITCH, src, 4);
@@ -137,7 +159,12 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
                 }
                 continue;
             }
-            const bool in = x9 >= 0 && x9 < W2 * 9;
+            const int j = min(max((col - 2) >> 1, 0), PWT - 1);
+            int b = b0, cj = c0 + j;
+            wrap(b, cj);
+            const int x = 2 * (cj - j) + col - 2, y0 = 2 * PH * b - 3;
+            const float* src = d2 + ((long long)y0 * W2 + x) * 9 + c;
+            const bool in = x >= 0 && x < W2;
 #pragma unroll 4
             for (int r = 0; r < HROWS; r++) {
                 const int y = y0 + r;
@@ -152,11 +179,11 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
 
     float* left = left_s + warp * NP * LEFT;             // this warp's: the last column of the tile before
     float* even = sm;                                    // the tile's buffer
-    if (B::BUFS == 2) stage(t, ry0, even);
+    if (B::BUFS == 2) stage(b0, c0, even);
 
     for (; todo > 0; todo--) {
-        const int cy0 = 2 * ry0 - 1;                     // first C0 row (may be -1)
-        if (B::BUFS == 1) stage(t, ry0, even);
+        const int cy0 = 2 * PH * b0 - 1;                 // lane 0's first C0 row (may be -1)
+        if (B::BUFS == 1) stage(b0, c0, even);
         if (load) {
             // (every warp has used the vectors before: with two buffers only the barrier here says so)
             if (B::BUFS == 2) __syncthreads();
@@ -187,20 +214,18 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
         }
         if (edged)
             for (int k = tid; k < 9 * HROWS; k += 256) {
-                const int c = k / HROWS, y = cy0 - 2 + k % HROWS;
-                const bool in = y >= 0 && y < H2;
-                cp_async4(edge + k, in ? d2 + ((long long)y * W2 + 2 * PWT * t - 3) * 9 + c : d2, in ? 4 : 0);
+                const int c = k / HROWS, x = 2 * c0 - 3, y = cy0 - 2 + k % HROWS;
+                const bool in = x >= 0 && y >= 0 && y < H2;
+                cp_async4(edge + k, in ? d2 + ((long long)y * W2 + x) * 9 + c : d2, in ? 4 : 0);
             }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
 
         // the tile after this one is staged while this one is computed
-        int tn = t + 1, yn = ry0;
-        if (tn == tiles) {
-            tn = 0;
-            yn = ry0 + PH < mh ? ry0 + PH : 0;
-        }
-        if (B::BUFS == 2 && todo > 1) stage(tn, yn, even == sm ? sm + 2 * COPY : sm);
+        int bn = b0, cn = c0 + PWT;
+        wrap(bn, cn);
+        if (++t == tiles) t = bn = cn = 0;
+        if (B::BUFS == 2 && todo > 1) stage(bn, cn, even == sm ? sm + 2 * COPY : sm);
 
         if (edged) {
             edged = false;
@@ -275,8 +300,10 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
         }
         if (B::BUFS == 1) __syncthreads();   // the next tile's descriptors may be staged
 
-        const int x = 2 * (PWT * t + lane), rx = PWT * t + lane;
-        const bool inner = 2 * PWT * (t + 1) <= W2 && cy0 >= 0 && cy0 + CROWS <= H2;
+        int band = b0, rx = c0 + lane;
+        wrap(band, rx);
+        const int x = 2 * rx, ry0 = band * PH;
+        const bool inner = 2 * (c0 + PWT) <= W2 && cy0 >= 0 && cy0 + CROWS <= H2;
         const long long pstride = (long long)mh * pitch;
 #pragma unroll
         for (int q = 0; q < NP; q++) {
@@ -286,7 +313,7 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
             if (!inner) {
 #pragma unroll
                 for (int r = 0; r < CROWS; r++) {
-                    const bool rin = cy0 + r >= 0 && cy0 + r < H2;
+                    const bool rin = 2 * ry0 - 1 + r >= 0 && 2 * ry0 - 1 + r < H2;
                     if (!(rin && x < W2)) v[r].x = -INFINITY;
                     if (!(rin && x + 1 < W2)) v[r].y = -INFINITY;
                 }
@@ -306,7 +333,7 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
             float* lq = left + q * LEFT;
             if (lane == 0) {
 #pragma unroll
-                for (int i = 0; i < PH; i++) before[i] = t > 0 ? lq[i] : -INFINITY;
+                for (int i = 0; i < PH; i++) before[i] = c0 > 0 ? lq[i] : -INFINITY;
                 yb = __float_as_uint(lq[8]);
             }
             __syncwarp();
@@ -346,40 +373,40 @@ k_corr0_f32(DmGeom g, const float* __restrict__ d1, const float* __restrict__ d2
                 o += 2 * pitch;
             }
         }
-        if (tn == 0 && yn == 0) p_base += PATCHES, load = true;
-        t = tn;
-        ry0 = yn;
+        if (t == 0) p_base += PATCHES, load = true;
+        b0 = bn;
+        c0 = cn;
         if (B::BUFS == 2) even = even == sm ? sm + 2 * COPY : sm;
     }
 }
 
 template <int PH, int NP>
-long long band_units(const DmGeom& g, int n_rows) {
+long long band_units(const DmGeom& g, int n_rows, int bl) {
     constexpr int P = Band<PH, NP>::PATCHES;
-    return (long long)((n_rows + P - 1) / P) * ((g.dh[1] + PH - 1) / PH) * ((g.dw[1] + PWT - 1) / PWT);
+    return (long long)((n_rows + P - 1) / P) * band_tiles((g.dh[1] + PH - 1) / PH, bl);
 }
 
 // The time of a form: tiles of the busiest SM, each its C0 rows and what costs about four
 // more of them besides, for the patches of a CTA; a quarter more where the CTAs of small
 // inputs begin inside a band, at a window that needs a column of its own.
 template <int PH, int NP>
-long long band_cost(const DmGeom& g, int n_rows) {
-    const long long c = (band_units<PH, NP>(g, n_rows) + SMS - 1) / SMS * (2 * PH + 5) * NP;
-    return NP == 2 && g.dw[1] > PWT ? c + c / 4 : c;
+long long band_cost(const DmGeom& g, int n_rows, int bl) {
+    const long long c = (band_units<PH, NP>(g, n_rows, bl) + SMS - 1) / SMS * (2 * PH + 5) * NP;
+    return NP == 2 && bl != PWT ? c + c / 4 : c;
 }
 
 template <int PH, int NP>
 cudaError_t launch_band(const DmGeom& g, const float* d1, const float* d2, float lam, float* pooled0, unsigned char* amax0,
-                        cudaStream_t st, const float* amat, int n_rows) {
+                        cudaStream_t st, const float* amat, int n_rows, int bl) {
     using B = Band<PH, NP>;
     static std::atomic<unsigned long long> smem_done{0};   // > 48 KB dynamic shared memory opted in, per device
     cudaError_t e = dm_smem_opt_in(reinterpret_cast<const void*>(k_corr0_f32<PH, NP>), (int)B::SMEM_BYTES, smem_done);
     if (e != cudaSuccess) return e;
-    const long long units = band_units<PH, NP>(g, n_rows), slots = SMS * B::CTAS_SM;
+    const long long units = band_units<PH, NP>(g, n_rows, bl), slots = SMS * B::CTAS_SM;
     const long long waves = (units + slots * RANGE - 1) / (slots * RANGE);
     const long long grid = units < slots ? units : slots * waves;
     e = dm_launch_pdl(k_corr0_f32<PH, NP>, (unsigned)grid, 256, B::SMEM_BYTES, st, g, d1, d2, lam, pooled0, amax0, amat, n_rows,
-                      units);
+                      units, bl);
     if (e != cudaSuccess) return e;
     dm_count_launches(1);
     return cudaGetLastError();
@@ -393,9 +420,20 @@ cudaError_t dm_launch_corr0_f32(const DmGeom& g, const float* d1, const float* d
     // The form with the shortest way: bands of 8 rows do the least extra work (17 C0 rows for
     // 16, against 9 for 8 and 5 for 4) and are taken by all but inputs of few tiles, whose
     // time is that of the busiest SM (64x48: 15.2 us with bands of 2, 29.5 with 8; 128x96: 83 us
-    // with 8 rows and 4 patches, 88 with 2 patches).
-    const long long c8 = band_cost<8, 4>(g, n_rows), c4 = band_cost<4, 2>(g, n_rows), c2 = band_cost<2, 2>(g, n_rows);
-    if (c8 <= c4 && c8 <= c2) return launch_band<8, 4>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows);
-    if (c4 <= c2) return launch_band<4, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows);
-    return launch_band<2, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows);
+    // with 8 rows and 4 patches, 88 with 2 patches).  Lanes of a band: whole tiles, or its
+    // columns and one (see above), where that makes the tiles fewer.
+    const int whole = (g.dw[1] + PWT - 1) / PWT * PWT, dense = g.dw[1] + 1;
+    int ph = 0, bl = 0;
+    long long best = 0;
+    auto consider = [&](int rows, int lanes, long long cost) {
+        if (ph == 0 || cost < best) ph = rows, bl = lanes, best = cost;
+    };
+    for (int lanes : {whole, dense}) {
+        consider(8, lanes, band_cost<8, 4>(g, n_rows, lanes));
+        consider(4, lanes, band_cost<4, 2>(g, n_rows, lanes));
+        consider(2, lanes, band_cost<2, 2>(g, n_rows, lanes));
+    }
+    if (ph == 8) return launch_band<8, 4>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows, bl);
+    if (ph == 4) return launch_band<4, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows, bl);
+    return launch_band<2, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows, bl);
 }

@@ -47,3 +47,12 @@ def test_level0_bit_exact(one, two, levels):
     np.testing.assert_array_equal(e, ex)
     np.testing.assert_array_equal(a, codes)
     np.testing.assert_array_equal(v.view(np.uint32), np.asarray(want, dtype=np.float32).view(np.uint32))
+
+
+# narrow maps and remainders: bands side by side in one row of tiles, each followed by an empty lane
+@pytest.mark.parametrize("levels", [2, 0])
+@pytest.mark.parametrize("one,two", [((256, 130), (24, 200)), ((130, 70), (5, 90)), ((257, 121), (62, 41)), ((300, 124), (64, 66)),
+                                     ((300, 124), (66, 64)), ((97, 75), (9, 7)), ((196, 193), (127, 60)), ((64, 48), (4, 301)),
+                                     ((220, 170), (200, 33))])
+def test_dense_bands_bit_exact(one, two, levels):
+    test_level0_bit_exact(one, two, levels)
