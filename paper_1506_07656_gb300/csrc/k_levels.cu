@@ -882,7 +882,7 @@ cudaError_t launch_rows(const DmGeom& g, int l, const dm_pyramid& py, const LvSh
 // they fill its strips (one of 64 or of 32) to 88 % or the image is small (the tiled
 // kernel's per-patch pipeline is then latency-bound; not where another tile than the default
 // was set, which is a request for it); for wider maps where they fill strips of 64 to
-// 88 % and the patches are enough to hide its loads: it moves less through L1 and L2 than
+// 88 % and the patches (twice the columns) are enough to hide its loads: it moves less through L1 and L2 than
 // the tiled kernel, which has no such granularity.  A fault-injection run takes the
 // tiled kernel, which holds the bounded waits.
 //   Measured (us, tiled / row-streaming; columns of the stored map in front): 1024x436 256
@@ -891,14 +891,14 @@ cudaError_t launch_rows(const DmGeom& g, int l, const dm_pyramid& py, const LvSh
 // 80 807 / 909, 20 80 / 115, 1242x375 156 1535 / 1790; 130x70 33 41 / 29.
 //   Image 1 of few patches (what the tiled kernel adds to a call of dm_correlate_pyramid): maps
 // of 40 columns, patches in front: 144 +9, 576 +10, 1024 +11, 1936 +13; 80 columns: 144 -15,
-// 576 -24, 1024 -29, 1936 -21; 160: -42, -38, -41, -48; 256 (filled): 144 -19, 576 +11, 1024
-// +28; 311 (filled): 144 -36, 400 -26, 576 -14, 1024 +1, 1936 +28.
+// 576 -24, 1024 -29, 1936 -21; 160: -42, -38, -41, -48; 128 (filled): 144 -2, 576 +8, 1024 +2;
+// 256 (filled): 144 -19, 576 +11, 1024 +28; 311 (filled): 144 -36, 400 -26, 576 -14, 1024 +1, 1936 +28.
 bool level_streams(const DmGeom& g, int l, const DmTune& tune, const LvShape& s) {
     const int ow = g.dw[l + 1], np = g.npatch(l);
     if (tune.level_th == 0 || ow <= 16) return true;
     const bool filled = s.fill >= 0.88, default_tile = tune.level_th == 8 && tune.level_ring == 2;
     if (ow <= 64) return (np <= 2048 && default_tile) || (filled && (s.lpp == 32 || ow <= 32));
-    return filled && s.lpp == 32 && np >= 512;
+    return filled && s.lpp == 32 && np >= 2 * ow;
 }
 
 // ---------------------------------------------------------------------------

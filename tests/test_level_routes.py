@@ -34,8 +34,9 @@ def tiled():
     # image 1 of 144 and 1936 patches, maps of 160, 80, 40 and 20 columns
     ((48, 48, 640, 480), SMALL, [1, 2]), ((176, 176, 640, 480), SMALL, [1, 2]), ((48, 48, 320, 240), SMALL, [1]),
     ((48, 48, 640, 480), (0, 2), []),
-    # filled maps of 311 and 256 columns: streaming from 512 patches on
-    ((48, 48, 1242, 375), SMALL, [1, 2, 3]), ((96, 96, 1242, 375), SMALL, [2, 3]), ((96, 96, 1024, 436), SMALL, []),
+    # filled maps of 311, 256 and 128 columns: streaming with twice as many patches
+    ((48, 48, 1242, 375), SMALL, [1, 2, 3]), ((96, 96, 1242, 375), SMALL, [1, 2, 3]), ((128, 128, 1242, 375), SMALL, [2, 3]),
+    ((96, 96, 1024, 436), SMALL, []), ((100, 75, 512, 224), SMALL, []),
     # as many patches as image 2 asks for
     ((1024, 436, 1024, 436), SMALL, []), ((1024, 436, 1024, 436), (16, 3), []), ((512, 224, 512, 224), SMALL, []),
     ((640, 480, 640, 480), SMALL, [1, 2, 3, 4]), ((1242, 375, 1242, 375), SMALL, [2, 3, 4, 5]),
