@@ -564,6 +564,15 @@ inline cudaError_t dm_prefer_l1(const void* kernel, std::atomic<unsigned long lo
     return e;
 }
 
+// SMs of the current device (152 on a whole GB300, fewer on a partition): grids and rules that
+// fill the GPU ask for it.
+inline int dm_sm_count() {
+    int dev = 0, nsm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return nsm;
+}
+
 // Launch with programmatic dependence on the kernel before it in the stream: its blocks
 // may become resident while that kernel's last ones run, which hides the launch (a
 // match at 64x48, 16 short kernels in a chain: 146 -> 110 us; a 319x237 pyramid 714 -> 679;

@@ -563,10 +563,7 @@ cudaError_t dm_launch_loss_grad(const DmGeom& g, const dm_pyramid& py, const flo
     em = cudaMemsetAsync(ws + gl.dP[0], 0, gl.dP[L - 1] + (size_t)g.npatch(L - 1) * g.psize(L) * 4 - gl.dP[0], st);
     if (em == cudaSuccess) em = cudaMemsetAsync(box0, 0x7f, (size_t)g.npatch(0) * sizeof(int4), st);
     if (em != cudaSuccess) return em;
-    int dev = 0, nsm = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned int fgrid = (unsigned int)nsm * 8;
+    const unsigned int fgrid = (unsigned int)dm_sm_count() * 8;
     for (int l = L; l >= 1; l--) {
         k_adj_down<<<fgrid, 256, 0, st>>>(g, l, py.valid[l], py.valid[l - 1], reinterpret_cast<const float*>(ws + gl.dA[l]),
                                           reinterpret_cast<float*>(ws + gl.dP[l - 1]), E, cnt + 2 * l, F,

@@ -728,13 +728,6 @@ BtArgs make_bt_args(const DmGeom& g, const dm_pyramid& py, const DmBtLayout& bl,
     return a;
 }
 
-int sm_count() {
-    int dev = 0, nsm = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    return nsm;
-}
-
 // Cross-pair form: the pairs of a wave of the batched form in one launch per
 // step, pair blockIdx.y (a cluster of blockIdx.x for the reciprocal step), its arguments in
 // the kernel parameters (a captured graph replays them as they were).  Step s
@@ -781,7 +774,7 @@ cudaError_t dm_launch_backtrack(const DmGeom& g, const dm_pyramid& py, const DmB
                                 dm_match_t* out, int capacity, int* d_count, cudaStream_t st, const DmRect* rect) {
     BtArgs a = make_bt_args(g, py, bl, ws);
     if (rect) a.rect = *rect;
-    const int grid = sm_count() * (py.tune.bt_mult > 0 ? py.tune.bt_mult : 8);
+    const int grid = dm_sm_count() * (py.tune.bt_mult > 0 ? py.tune.bt_mult : 8);
     if (rect) {
         launch_steps<BT_RECT>(a, grid, st);
         return cudaGetLastError();
@@ -824,9 +817,7 @@ cudaError_t dm_launch_backtrack_star(const DmGeom& g, const dm_pyramid& py, cons
     const size_t ncell = (size_t)((g.W2 + 3) / 4) * ((g.H2 + 3) / 4);
     if ((e = cudaMemsetAsync(a.bestQ, 0, sizeof(unsigned long long) * ncell, st)) != cudaSuccess) return e;
 
-    int dev = 0, nsm = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int nsm = dm_sm_count();
     const int grid = nsm * (py.tune.bt_mult > 0 ? py.tune.bt_mult : 8);
     auto items = [&](int l) -> long long {
         return (long long)g.npatch(l) * ((g.dw[l] + ST_COLS - 1) / ST_COLS) * ((g.dh[l] + ST_ROWS - 1) / ST_ROWS);
@@ -886,7 +877,7 @@ cudaError_t dm_launch_backtrack_batch(const dm_pyramid* const* pys, const DmBtLa
         Lmax = max(Lmax, pys[j]->g.L);
         if (pys[j]->tune.bt_mult > 0) mult = pys[j]->tune.bt_mult;
     }
-    const int nsm = sm_count();
+    const int nsm = dm_sm_count();
     // blocks per pair: the single-pair grid shared by the wave, at least one per SM
     const int per = max(nsm, nsm * mult / n);
     long long launches = 0;

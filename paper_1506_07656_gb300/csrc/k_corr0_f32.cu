@@ -64,7 +64,6 @@ constexpr int PWT = 32;                       // pooled columns per tile
 constexpr int HCOLS = 2 * PWT + 3;            // pixels 64 t - 2 .. 64 t + 64
 constexpr int HPITCH = 66;                    // columns of a staged row (either copy)
 constexpr int LEFT = 12;                      // a patch's column kept for the next tile: 8 maxima, their rows, padding
-constexpr int SMS = 152;
 constexpr int RANGE = 32;                     // tiles of a CTA, at most
 
 // A band of PH pooled rows, NP patches per warp.
@@ -390,19 +389,19 @@ long long band_units(const DmGeom& g, int n_rows, int bl) {
 // more of them besides, for the patches of a CTA; a quarter more where the CTAs of small
 // inputs begin inside a band, at a window that needs a column of its own.
 template <int PH, int NP>
-long long band_cost(const DmGeom& g, int n_rows, int bl) {
-    const long long c = (band_units<PH, NP>(g, n_rows, bl) + SMS - 1) / SMS * (2 * PH + 5) * NP;
+long long band_cost(const DmGeom& g, int n_rows, int bl, int sms) {
+    const long long c = (band_units<PH, NP>(g, n_rows, bl) + sms - 1) / sms * (2 * PH + 5) * NP;
     return NP == 2 && bl != PWT ? c + c / 4 : c;
 }
 
 template <int PH, int NP>
 cudaError_t launch_band(const DmGeom& g, const float* d1, const float* d2, float lam, float* pooled0, unsigned char* amax0,
-                        cudaStream_t st, const float* amat, int n_rows, int bl) {
+                        cudaStream_t st, const float* amat, int n_rows, int bl, int sms) {
     using B = Band<PH, NP>;
     static std::atomic<unsigned long long> smem_done{0};   // > 48 KB dynamic shared memory opted in, per device
     cudaError_t e = dm_smem_opt_in(reinterpret_cast<const void*>(k_corr0_f32<PH, NP>), (int)B::SMEM_BYTES, smem_done);
     if (e != cudaSuccess) return e;
-    const long long units = band_units<PH, NP>(g, n_rows, bl), slots = SMS * B::CTAS_SM;
+    const long long units = band_units<PH, NP>(g, n_rows, bl), slots = (long long)sms * B::CTAS_SM;
     const long long waves = (units + slots * RANGE - 1) / (slots * RANGE);
     const long long grid = units < slots ? units : slots * waves;
     e = dm_launch_pdl(k_corr0_f32<PH, NP>, (unsigned)grid, 256, B::SMEM_BYTES, st, g, d1, d2, lam, pooled0, amax0, amat, n_rows,
@@ -422,18 +421,18 @@ cudaError_t dm_launch_corr0_f32(const DmGeom& g, const float* d1, const float* d
     // time is that of the busiest SM (64x48: 15.2 us with bands of 2, 29.5 with 8; 128x96: 83 us
     // with 8 rows and 4 patches, 88 with 2 patches).  Lanes of a band: whole tiles, or its
     // columns and one (see above), where that makes the tiles fewer.
-    const int whole = (g.dw[1] + PWT - 1) / PWT * PWT, dense = g.dw[1] + 1;
+    const int whole = (g.dw[1] + PWT - 1) / PWT * PWT, dense = g.dw[1] + 1, sms = dm_sm_count();
     int ph = 0, bl = 0;
     long long best = 0;
     auto consider = [&](int rows, int lanes, long long cost) {
         if (ph == 0 || cost < best) ph = rows, bl = lanes, best = cost;
     };
     for (int lanes : {whole, dense}) {
-        consider(8, lanes, band_cost<8, 4>(g, n_rows, lanes));
-        consider(4, lanes, band_cost<4, 2>(g, n_rows, lanes));
-        consider(2, lanes, band_cost<2, 2>(g, n_rows, lanes));
+        consider(8, lanes, band_cost<8, 4>(g, n_rows, lanes, sms));
+        consider(4, lanes, band_cost<4, 2>(g, n_rows, lanes, sms));
+        consider(2, lanes, band_cost<2, 2>(g, n_rows, lanes, sms));
     }
-    if (ph == 8) return launch_band<8, 4>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows, bl);
-    if (ph == 4) return launch_band<4, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows, bl);
-    return launch_band<2, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows, bl);
+    if (ph == 8) return launch_band<8, 4>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows, bl, sms);
+    if (ph == 4) return launch_band<4, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows, bl, sms);
+    return launch_band<2, 2>(g, d1, d2, lam, pooled0, amax0, st, amat, n_rows, bl, sms);
 }

@@ -701,17 +701,10 @@ bool make_map(CUtensorMap* m, void* base, CUtensorMapDataType dt, int esize, con
     return dm_encode_tiled(m, dt, 3, base, dims, strides, box, sw);
 }
 
-int tc_sm_count() {
-    int dev = 0, nsm = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    return nsm;
-}
-
 template <int FMT>
 cudaError_t launch_tc(const L0Batch& B, float lam, cudaStream_t st) {
     using F = Fmt<FMT>;
-    const int nsm = tc_sm_count();
+    const int nsm = dm_sm_count();
     static std::atomic<unsigned long long> smem_done{0};
     cudaError_t ea = dm_smem_opt_in(reinterpret_cast<const void*>(k_corr0_tc<FMT>), (int)F::SMEM, smem_done);
     if (ea != cudaSuccess) return ea;
@@ -734,7 +727,7 @@ cudaError_t prepare_pair(const DmGeom& g, int precision, const float* d1, const 
     // (tiles + about one tile's time for the unit's operand), by 2 % or more (256x256
     // BF16: one chunk of 32 tiles 263 us, this choice 209; the choice does not depend on
     // whether half a tile or three stand for the operand).
-    const int pairs = ((g.dw[1] + SX - 1) / SX) * ((g.dh[1] + PY - 1) / PY), nsm = tc_sm_count();
+    const int pairs = ((g.dw[1] + SX - 1) / SX) * ((g.dh[1] + PY - 1) / PY), nsm = dm_sm_count();
     if (m_chunk < 1) m_chunk = 1;
     int best = 0;
     double best_cost = 0.0;
@@ -763,8 +756,8 @@ cudaError_t prepare_pair(const DmGeom& g, int precision, const float* d1, const 
         unsigned int* bmax = reinterpret_cast<unsigned int*>(apack + a_bytes + dm_align((size_t)n_mtiles * BM * sizeof(float)));
         if ((e = cudaMemsetAsync(bmax, 0, sizeof(unsigned int), st)) != cudaSuccess) return e;
         const long long n2 = (long long)g.W2 * g.H2 * 9;
-        const long long blocks = (n2 / 4 + 255) / 256;
-        k_absmax<<<(unsigned)(blocks < 1216 ? (blocks > 0 ? blocks : 1) : 1216), 256, 0, st>>>(d2, n2, bmax);
+        const long long blocks = std::min<long long>((n2 / 4 + 255) / 256, 8LL * dm_sm_count());
+        k_absmax<<<(unsigned)(blocks > 0 ? blocks : 1), 256, 0, st>>>(d2, n2, bmax);
         k_pack_a8<<<(unsigned)((n_mtiles * BM + 127) / 128), 128, 0, st>>>(g, d1, apack, inv_sa, n_mtiles, amat, n0);
         q->inv_sa = inv_sa;
         q->bmax = bmax;

@@ -389,7 +389,7 @@ cudaError_t launch_fused(const DmDescParams& prm, const Taps7 t[3], const IoBatc
 cudaError_t launch_fused(const DmDescParams& prm, const Taps7 t[3], const IoBatch& b, cudaStream_t st) {
     long long px = 0;
     for (int i = 0; i < b.n; i++) px += (long long)b.W[i] * b.H[i];
-    if (px >= 32 * 16 * 152) return launch_fused<32, 16>(prm, t, b, st);
+    if (px >= 32LL * 16 * dm_sm_count()) return launch_fused<32, 16>(prm, t, b, st);
     return launch_fused<16, 8>(prm, t, b, st);
 }
 

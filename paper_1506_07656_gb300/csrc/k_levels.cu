@@ -831,7 +831,7 @@ struct LvShape {
     long long blocks;
 };
 
-LvShape level_shape(const DmGeom& g, int l) {
+LvShape level_shape(const DmGeom& g, int l, int sms) {
     LvShape s;
     const int ow = g.dw[l + 1], oh = g.dh[l + 1], S = level_stride(l);
     // lanes per unit: the least lanes per row, a unit's memory sectors past its edges
@@ -852,7 +852,8 @@ LvShape level_shape(const DmGeom& g, int l) {
     // whole columns 6.34, 64 rows 6.34, 32 rows 6.34, 16 rows 6.50 ms for the levels of
     // 1024x436), shorter where the patches alone leave the GPU idle
     const long long per_seg = (long long)S * s.nby * strips * ((S * s.nbx + LV_GROUP - 1) / LV_GROUP) * LV_GROUP;
-    const long long segs = std::max<long long>((oh + 31) / 32, std::min<long long>((oh + 2) / 3, (1216 + per_seg - 1) / per_seg));
+    const long long fit = 8LL * sms;
+    const long long segs = std::max<long long>((oh + 31) / 32, std::min<long long>((oh + 2) / 3, (fit + per_seg - 1) / per_seg));
     s.seg_rows = (int)((oh + segs - 1) / segs);
     s.blocks = (long long)((oh + s.seg_rows - 1) / s.seg_rows) * per_seg;
     return s;
@@ -984,18 +985,19 @@ __global__ void k_level_top_b(const __grid_constant__ LvBatch B, int l, float la
 }  // namespace
 
 bool dm_level_tiled(const DmGeom& g, int l, const DmTune& tune) {
-    return l >= 1 && l < g.L && !level_streams(g, l, tune, level_shape(g, l));
+    return l >= 1 && l < g.L && !level_streams(g, l, tune, level_shape(g, l, 1));   // (the rule does not depend on the SMs)
 }
 
 cudaError_t dm_launch_levels(const DmGeom& g, const dm_pyramid& py, float lam, int* status, cudaStream_t st) {
     const int B = 128;
     int n0 = g.npatch(0), np = g.npatch(1);
+    const int sms = dm_sm_count();
     const bool whole = valid_fits(g);
     if (whole) dm_launch_pdl(k_valid_all, valid_blocks(max(n0, np)), VALID_THREADS, 0, st, valid_args(py));
     else k_fill_u8<<<(n0 + 255) / 256, 256, 0, st>>>(const_cast<unsigned char*>(py.valid[0]), n0, 1);
     for (int l = 1; l <= g.L; l++) {
         if (!whole) k_valid<<<(np + 255) / 256, 256, 0, st>>>(g, l, py.valid[l - 1], const_cast<unsigned char*>(py.valid[l]));
-        const LvShape sh = l < g.L ? level_shape(g, l) : LvShape();
+        const LvShape sh = l < g.L ? level_shape(g, l, sms) : LvShape();
         if (l < g.L && py.inject_wait == 0 && level_streams(g, l, py.tune, sh)) {
             const cudaError_t e = py.compensated ? launch_rows<true>(g, l, py, sh, lam, st) : launch_rows<false>(g, l, py, sh, lam, st);
             if (e != cudaSuccess) return e;
@@ -1053,6 +1055,7 @@ cudaError_t dm_launch_levels(const DmGeom& g, const dm_pyramid& py, float lam, i
 cudaError_t dm_launch_levels_batch(const dm_pyramid* const* pys, int n, float lam, int* const* status, cudaStream_t st) {
     if (n < 1 || n > DM_BATCH_MAX) return cudaErrorInvalidValue;
     const bool comp = pys[0]->compensated != 0;
+    const int sms = dm_sm_count();
     int Lmax = 0;
     for (int j = 0; j < n; j++) Lmax = max(Lmax, pys[j]->g.L);
     long long launches = 0;
@@ -1126,7 +1129,7 @@ cudaError_t dm_launch_levels_batch(const dm_pyramid* const* pys, int n, float la
                 const dm_pyramid& py = *pys[j];
                 const DmGeom& g = py.g;
                 if (l >= g.L) continue;
-                const LvShape sh = level_shape(g, l);
+                const LvShape sh = level_shape(g, l, sms);
                 const bool stream = level_streams(g, l, py.tune, sh);
                 const int th = py.tune.level_th == 8 || py.tune.level_th == 4 ? py.tune.level_th : 16;
                 const int nr = py.tune.level_ring == 3 ? 3 : 2;
