@@ -364,8 +364,8 @@ __device__ __forceinline__ void dm_two_sum2(float2& s, float2 x, float2& err) {
 
 // Average of four children's values, two columns per packed FP32x2 operation (a missing child's are
 // zeros, which leave both the plain and the compensated sum of the others unchanged: s + 0 = s
-// exactly, with a zero TwoSum error): times w (1/n for n = 1, 2, 4, exact) or, for n = 3, divided by 3.
-template <bool COMP, bool DIV3>
+// exactly, with a zero TwoSum error), times w = 1/n (n is 1, 2 or 4, so exact).
+template <bool COMP>
 __device__ __forceinline__ float2 avg_pair4(float2 x0, float2 x1, float2 x2, float2 x3, float w) {
     float2 sv = x0;
     if constexpr (COMP) {
@@ -381,7 +381,7 @@ __device__ __forceinline__ float2 avg_pair4(float2 x0, float2 x1, float2 x2, flo
     } else {
         sv = __fadd2_rn(__fadd2_rn(__fadd2_rn(sv, x1), x2), x3);
     }
-    return DIV3 ? make_float2(__fdiv_rn(sv.x, 3.0f), __fdiv_rn(sv.y, 3.0f)) : __fmul2_rn(sv, make_float2(w, w));
+    return __fmul2_rn(sv, make_float2(w, w));
 }
 
 // One step of the compensated child sum (Knuth's TwoSum gives the same bits

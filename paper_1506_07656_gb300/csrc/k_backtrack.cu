@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(256, 4) k_star_entries(BtArgs a, int l, float 
             r.v = make_float2(-INFINITY, -INFINITY);
             if (y >= 0 && y < mh) {                    // the same for the whole warp, as is k.n
                 if (k.n == 4) {
-                    r.v = avg_pair4<COMP, false>(pair(0, y), pair(1, y), pair(2, y), pair(3, y), 0.25f);
+                    r.v = avg_pair4<COMP>(pair(0, y), pair(1, y), pair(2, y), pair(3, y), 0.25f);
                     if (!in0) r.v.x = -INFINITY;
                     if (!in1) r.v.y = -INFINITY;
                 } else {

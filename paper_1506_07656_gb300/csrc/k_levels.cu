@@ -41,9 +41,10 @@ namespace {
 
 // valid[l][p] = 1 iff some child exists (Eq. 7 with the boundary rule; level 0: every
 // atomic patch).  A patch's children are two columns times two rows, so it exists iff
-// its column and its row do: every CTA derives the columns' and rows' flags of all levels
-// in shared memory and writes its share of the patches, all levels in one launch (one
-// launch per level took 28 us at 1024x436 and, at 64x48, 15 of 157).
+// its column and its row do, and has 0, 1, 2 or 4 existing children, never 3.  Every CTA
+// derives the columns' and rows' flags of all levels in shared memory and writes its share of
+// the patches, all levels in one launch (one launch per level took 28 us at 1024x436 and, at
+// 64x48, 15 of 157).
 constexpr int VALID_SIDE = 8192;             // lattice columns + rows of a pair, at most; larger ones level by level
 constexpr int VALID_THREADS = 1024;
 struct ValidArgs {
@@ -153,26 +154,25 @@ constexpr long long LEVEL_WAIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
 // Children with o_x = -1 (left, windows lt / lb) read columns ax+2 .. ax+5 (two
 // aligned float4 loads, which unlike 8-byte loads at a 16-byte stride are free
 // of bank conflicts), children with o_x = +1 (right, rt / rb) columns
-// ax+4 .. ax+7.  Then times w (1/n for n = 1, 2, 4, exact) or, for n = 3,
-// divided by 3.  Two columns per packed FP32x2 operation: Knuth's TwoSum (6
+// ax+4 .. ax+7.  Then times w = 1/n (n is 1, 2 or 4: valid_all).  Two columns per packed FP32x2 operation: Knuth's TwoSum (6
 // additions, every step correctly rounded per lane) costs 3 instructions per
 // column and step.
-template <bool COMP, bool DIV3>
+template <bool COMP>
 __device__ __forceinline__ float4 avg_group(const float* lt, const float* lb, const float* rt, const float* rb, float w) {
     const float4 a0 = *reinterpret_cast<const float4*>(lt), b0 = *reinterpret_cast<const float4*>(lt + 4);
     const float4 a1 = *reinterpret_cast<const float4*>(lb), b1 = *reinterpret_cast<const float4*>(lb + 4);
     const float4 v2 = *reinterpret_cast<const float4*>(rt + 4);
     const float4 v3 = *reinterpret_cast<const float4*>(rb + 4);
-    const float2 r0 = avg_pair4<COMP, DIV3>(make_float2(a0.z, a0.w), make_float2(a1.z, a1.w), make_float2(v2.x, v2.y),
+    const float2 r0 = avg_pair4<COMP>(make_float2(a0.z, a0.w), make_float2(a1.z, a1.w), make_float2(v2.x, v2.y),
                                             make_float2(v3.x, v3.y), w);
-    const float2 r1 = avg_pair4<COMP, DIV3>(make_float2(b0.x, b0.y), make_float2(b1.x, b1.y), make_float2(v2.z, v2.w),
+    const float2 r1 = avg_pair4<COMP>(make_float2(b0.x, b0.y), make_float2(b1.x, b1.y), make_float2(v2.z, v2.w),
                                             make_float2(v3.z, v3.w), w);
     return make_float4(r0.x, r0.y, r1.x, r1.y);
 }
 
 // The same for two columns c, c+1 (c even: 8-byte loads at columns c+2 and
 // c+4), or -- ONE -- for column c alone (the second lane's result unused).
-template <bool COMP, bool DIV3, bool ONE>
+template <bool COMP, bool ONE>
 __device__ __forceinline__ float2 avg_two(const float* lt, const float* lb, const float* rt, const float* rb, float w) {
     float2 x[4];
     if constexpr (ONE) {
@@ -186,7 +186,7 @@ __device__ __forceinline__ float2 avg_two(const float* lt, const float* lb, cons
         x[2] = *reinterpret_cast<const float2*>(rt + 4);
         x[3] = *reinterpret_cast<const float2*>(rb + 4);
     }
-    return avg_pair4<COMP, DIV3>(x[0], x[1], x[2], x[3], w);
+    return avg_pair4<COMP>(x[0], x[1], x[2], x[3], w);
 }
 
 // Sweep geometry of level l: a CTA owns one tile of TW x TH pooled outputs of a
@@ -374,8 +374,7 @@ __device__ __forceinline__ void level_sweep_body(const DmGeom& g, int l, const C
                 const int e = tid + u * NT;
                 const int ay = e >> 4, ax = 4 * (e & 15);
                 const int o = ay * KW + ax;
-                float4 a = n == 3 ? avg_group<COMP, true>(lt + o, lt + KIDF + o, rt + o, rt + KIDF + o, w)
-                                  : avg_group<COMP, false>(lt + o, lt + KIDF + o, rt + o, rt + KIDF + o, w);
+                float4 a = avg_group<COMP>(lt + o, lt + KIDF + o, rt + o, rt + KIDF + o, w);
                 if (!interior) {
                     mask(a.x, ay, ax);
                     mask(a.y, ay, ax + 1);
@@ -390,8 +389,7 @@ __device__ __forceinline__ void level_sweep_body(const DmGeom& g, int l, const C
                 if (x < 32) {
                     // last row, columns 2x, 2x + 1
                     const int ay = AH - 1, ax = 2 * x, o = ay * KW + ax;
-                    float2 a = n == 3 ? avg_two<COMP, true, false>(lt + o, lt + KIDF + o, rt + o, rt + KIDF + o, w)
-                                      : avg_two<COMP, false, false>(lt + o, lt + KIDF + o, rt + o, rt + KIDF + o, w);
+                    float2 a = avg_two<COMP, false>(lt + o, lt + KIDF + o, rt + o, rt + KIDF + o, w);
                     if (!interior) {
                         mask(a.x, ay, ax);
                         mask(a.y, ay, ax + 1);
@@ -400,8 +398,7 @@ __device__ __forceinline__ void level_sweep_body(const DmGeom& g, int l, const C
                 } else {
                     // column 64 of row x - 32
                     const int ay = x - 32, ax = AW - 1, o = ay * KW + ax;
-                    float2 a = n == 3 ? avg_two<COMP, true, true>(lt + o, lt + KIDF + o, rt + o, rt + KIDF + o, w)
-                                      : avg_two<COMP, false, true>(lt + o, lt + KIDF + o, rt + o, rt + KIDF + o, w);
+                    float2 a = avg_two<COMP, true>(lt + o, lt + KIDF + o, rt + o, rt + KIDF + o, w);
                     if (!interior) mask(a.x, ay, ax);
                     avg[ay][ax] = a.x;
                 }
@@ -718,8 +715,6 @@ __device__ __forceinline__ void level_rows_body(const DmGeom& g, int l, const fl
             n++;
         }
     }
-    // existence factorises into columns times rows (the four children are two
-    // columns times two rows, level by level), so n is 0, 1, 2 or 4
     L.w = n == 4 ? 0.25f : (n == 2 ? 0.5f : 1.0f);
     const bool any = __any_sync(0xffffffffu, n > 0);
     // every unit of the warp has all its children and a complete strip (and byte
