@@ -147,6 +147,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// A bounded wait of a kernel that gives up, for what it has in flight itself.
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+    const long long t0 = clock64();
+    uint32_t ok = 0;
+    while (!ok && clock64() - t0 <= WAIT_CYCLES)
+        asm volatile("{.reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p;}"
+                     : "=r"(ok) : "r"(bar), "r"(parity), "n"(WAIT_HINT_NS) : "memory");
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count) : "memory");
 }
@@ -471,6 +480,7 @@ struct L0Pair {
 struct L0Batch {
     L0Pair p[DM_BATCH_MAX];
     int n, total;
+    long long inject_wait;       // > 0 (dm_inject_fault): every CTA gives up after its first tile's MMAs
 };
 
 template <int FMT>
@@ -483,13 +493,14 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
     float* sF = reinterpret_cast<float*>(smem + F::OFF_F);
     unsigned char* sC = smem + F::OFF_C;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + F::OFF_BAR);
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 2 * F::STAGES + 9);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 2 * F::STAGES + 10);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
     const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + F::STAGES);
     const uint32_t bar_acc_full = smem_u32(bars + 2 * F::STAGES), bar_acc_empty = smem_u32(bars + 2 * F::STAGES + 2);
     // group b has staged its tile; the stores have read group b's values, the codes
     const uint32_t bar_staged = smem_u32(bars + 2 * F::STAGES + 4), bar_vfree = smem_u32(bars + 2 * F::STAGES + 6);
     const uint32_t bar_cfree = smem_u32(bars + 2 * F::STAGES + 8);
+    const uint32_t bar_gone = smem_u32(bars + 2 * F::STAGES + 9);    // giving up: every MMA issued is done
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
@@ -504,6 +515,7 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
             mbar_init(bar_vfree + 8 * b, 1);
         }
         mbar_init(bar_cfree, 1);
+        mbar_init(bar_gone, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -517,6 +529,7 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
 
     // tiles so far: A tiles (and stores), and those of accumulator 1
     uint32_t a_it = 0, acc1_it = 0;
+    uint32_t issued = 0;                             // copies of A that this thread has started
 
     for (int gu = blockIdx.x; gu < B.total; gu += gridDim.x) {
         int pj = 0;
@@ -584,6 +597,7 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
                     const unsigned char* src = apack + (long long)(m0 + j) * F::A_TILE;
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                                  :: "r"(smem_u32(sA + s * F::A_TILE)), "l"(src), "r"(F::A_TILE), "r"(bar_full + 8 * s) : "memory");
+                    issued = it + 1;
                 }
             }
         } else if (warp == 1) {
@@ -611,6 +625,17 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
                                              :: "r"(d_tmem), "l"(ad), "l"(bd), "r"(F::IDESC), "r"(acc) : "memory");
                         }
                         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar_acc_full + 8 * b) : "memory");
+                    }
+                    if (B.inject_wait > 0 && ok) {
+                        // fault injection: a bounded wait on a barrier nothing completes runs out
+                        const long long t0 = clock64();
+                        uint32_t done = 0;
+                        while (!done && clock64() - t0 <= B.inject_wait)
+                            asm volatile("{.reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p;}"
+                                         : "=r"(done) : "r"(bar_gone), "r"(0u), "n"(WAIT_HINT_NS) : "memory");
+                        atomicOr(err, 1);
+                        *abort_flag = 1;
+                        ok = false;
                     }
                     if (ok)
                         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar_empty + 8 * s) : "memory");
@@ -685,6 +710,17 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
         if (two) acc1_it += nt;
         __syncthreads();   // the epilogue has consumed every accumulator: the tensor core is done with sB
         if (*abort_flag) break;
+    }
+    if (*abort_flag) {
+        // a wait has run out: the copies of A and the MMAs still in flight end before shared memory and TMEM
+        // are given back (each wait bounded again)
+        if (warp == 0 && lane == 0)
+            for (uint32_t it = issued > F::STAGES ? issued - F::STAGES : 0; it < issued; it++)
+                mbar_drain(bar_full + 8 * (it % F::STAGES), (it / F::STAGES) & 1);
+        if (warp == 1 && lane == 0) {
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar_gone) : "memory");
+            mbar_drain(bar_gone, 0);
+        }
     }
     if (warp == STORE_WARP && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     __syncthreads();
@@ -805,12 +841,13 @@ size_t dm_corr0_tc_a_bytes(const DmGeom& g, int precision) {
 
 cudaError_t dm_launch_corr0_tc(const DmGeom& g, int precision, const float* d1, const float* d2, float lam, void* abuf,
                                void* status, float* pooled0, unsigned char* amax0, int m_chunk, cudaStream_t st,
-                               const float* amat, int n_rows) {
+                               const float* amat, int n_rows, long long inject_wait) {
     std::unique_ptr<L0Batch> B(new L0Batch);
     memset(B.get(), 0, sizeof(L0Batch));
     cudaError_t e = prepare_pair(g, precision, d1, d2, abuf, status, pooled0, amax0, m_chunk, st, amat, n_rows, &B->p[0]);
     if (e != cudaSuccess) return e;
     B->n = 1;
+    B->inject_wait = inject_wait;
     B->total = B->p[0].units;
     e = precision == DM_FP8_E4M3 ? launch_tc<FMT_E4M3>(*B, lam, st) : launch_tc<FMT_BF16>(*B, lam, st);
     dm_count_launches(1);
