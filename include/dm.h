@@ -335,17 +335,16 @@ dm_status dm_read_status(dm_ctx* ctx, const void* d_ws, int* status, long long* 
  *                      DM_DEV_FRONTIER_OVERFLOW (dm_read_status) and returns
  *                      the matches of the tuples that fitted.  arg = 0: off.
  *   DM_FAULT_WAIT      every CTA of the level kernel (levels 1..L-1) first
- *                      waits arg clock cycles on a barrier nothing completes, and
- *                      in BF16 and FP8 every CTA of the level-0 kernel (outside
- *                      waves of the batched form) after its first tile; the
- *                      bounded wait runs out, the CTA waits for the loads, MMAs
- *                      and stores it has started and exits, and dm_read_status
- *                      on the pyramid (or dm_match) workspace reports
- *                      DM_DEV_TIMEOUT; the pyramid's contents are then undefined.
- *                      arg = 0: off.
+ *                      waits arg clock cycles on a barrier nothing completes;
+ *                      the bounded wait runs out, the CTA waits for the loads
+ *                      it has started and exits, and dm_read_status on the
+ *                      pyramid (or dm_match) workspace reports DM_DEV_TIMEOUT;
+ *                      the pyramid's contents are then undefined.  arg = 0: off.
  *   DM_FAULT_ALLOC     process-wide (ctx may be NULL): the arg-th next resource
  *                      creation (dm_create's context, dm_timing_start's events)
- *                      fails with DM_ENOMEM and leaves nothing behind. */
+ *                      fails with DM_ENOMEM and leaves nothing behind.
+ * Not covered: a run-out of the tensor-core level-0 kernel's waits (it ends the
+ * copies and MMAs it has issued, reports DM_DEV_TIMEOUT and returns). */
 #define DM_FAULT_NONE 0
 #define DM_FAULT_LAUNCH 1
 #define DM_FAULT_CAPACITY 2

@@ -204,7 +204,7 @@ dm_status run_pyramid(dm_ctx* c, const DmGeom& g, const float* d1, const float* 
     if (c->cfg.precision != DM_FP32) {
         e = dm_launch_corr0_tc(g, c->cfg.precision, d1, d2, c->cfg.lambda, base + pl.a16, d_status,
                                const_cast<float*>(py->pooled[0]), const_cast<unsigned char*>(py->amax[0]),
-                               py->tune.m_chunk, st, protos, py->n0_maps, py->inject_wait);
+                               py->tune.m_chunk, st, protos, py->n0_maps);
     } else {
         e = dm_launch_corr0_f32(g, d1, d2, c->cfg.lambda, const_cast<float*>(py->pooled[0]),
                                 const_cast<unsigned char*>(py->amax[0]), st, protos, py->n0_maps);
@@ -739,7 +739,7 @@ dm_status dm_match(dm_ctx* ctx, const float* d_img1, int W1, int H1, const float
     if (ctx->cfg.precision != DM_FP32)
         e = dm_launch_corr0_tc(g, ctx->cfg.precision, desc1, desc2, ctx->cfg.lambda, base + ml.pyr + ml.py.a16,
                                d_status, const_cast<float*>(py.pooled[0]), const_cast<unsigned char*>(py.amax[0]),
-                               py.tune.m_chunk, st, nullptr, -1, py.inject_wait);
+                               py.tune.m_chunk, st);
     else
         e = dm_launch_corr0_f32(g, desc1, desc2, ctx->cfg.lambda, const_cast<float*>(py.pooled[0]),
                                 const_cast<unsigned char*>(py.amax[0]), st);

@@ -333,10 +333,9 @@ struct dm_pyramid {
     // exact form: proto_of = nullptr, n0_maps = npatch(0)
     const int* proto_of;
     int n0_maps;
-    // fault injection (dm_inject_fault): > 0, every CTA of the level kernel (and of
-    // the tensor-core level 0, after its first tile) waits this many cycles on a
-    // barrier nothing completes, so its bounded wait runs out and the pyramid status
-    // reports it; 0 otherwise
+    // fault injection (dm_inject_fault): > 0, every CTA of the level kernel
+    // first waits this many cycles on a barrier nothing completes, so its
+    // bounded wait runs out and the pyramid status reports it; 0 otherwise
     long long inject_wait;
 };
 
@@ -630,7 +629,7 @@ cudaError_t dm_launch_corr0_f32(const DmGeom& g, const float* d1, const float* d
 // dm_corr0_tc_a_bytes(g, precision) bytes of packed operands.
 cudaError_t dm_launch_corr0_tc(const DmGeom& g, int precision, const float* d1, const float* d2, float lam, void* abuf,
                                void* status, float* pooled0, unsigned char* amax0, int m_chunk, cudaStream_t st,
-                               const float* amat = nullptr, int n_rows = -1, long long inject_wait = 0);
+                               const float* amat = nullptr, int n_rows = -1);
 // Level 0 of the n <= DM_BATCH_MAX pairs of a wave (exact form): their operand
 // packing, then one persistent launch that drains the work units of all pairs.
 cudaError_t dm_launch_corr0_tc_batch(int n, const DmGeom* gs, int precision, const float* const* d1s,

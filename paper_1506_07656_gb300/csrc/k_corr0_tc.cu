@@ -480,7 +480,6 @@ struct L0Pair {
 struct L0Batch {
     L0Pair p[DM_BATCH_MAX];
     int n, total;
-    long long inject_wait;       // > 0 (dm_inject_fault): every CTA gives up after its first tile's MMAs
 };
 
 template <int FMT>
@@ -625,17 +624,6 @@ k_corr0_tc(const __grid_constant__ L0Batch B, float lam) {
                                              :: "r"(d_tmem), "l"(ad), "l"(bd), "r"(F::IDESC), "r"(acc) : "memory");
                         }
                         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar_acc_full + 8 * b) : "memory");
-                    }
-                    if (B.inject_wait > 0 && ok) {
-                        // fault injection: a bounded wait on a barrier nothing completes runs out
-                        const long long t0 = clock64();
-                        uint32_t done = 0;
-                        while (!done && clock64() - t0 <= B.inject_wait)
-                            asm volatile("{.reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p;}"
-                                         : "=r"(done) : "r"(bar_gone), "r"(0u), "n"(WAIT_HINT_NS) : "memory");
-                        atomicOr(err, 1);
-                        *abort_flag = 1;
-                        ok = false;
                     }
                     if (ok)
                         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar_empty + 8 * s) : "memory");
@@ -841,13 +829,12 @@ size_t dm_corr0_tc_a_bytes(const DmGeom& g, int precision) {
 
 cudaError_t dm_launch_corr0_tc(const DmGeom& g, int precision, const float* d1, const float* d2, float lam, void* abuf,
                                void* status, float* pooled0, unsigned char* amax0, int m_chunk, cudaStream_t st,
-                               const float* amat, int n_rows, long long inject_wait) {
+                               const float* amat, int n_rows) {
     std::unique_ptr<L0Batch> B(new L0Batch);
     memset(B.get(), 0, sizeof(L0Batch));
     cudaError_t e = prepare_pair(g, precision, d1, d2, abuf, status, pooled0, amax0, m_chunk, st, amat, n_rows, &B->p[0]);
     if (e != cudaSuccess) return e;
     B->n = 1;
-    B->inject_wait = inject_wait;
     B->total = B->p[0].units;
     e = precision == DM_FP8_E4M3 ? launch_tc<FMT_E4M3>(*B, lam, st) : launch_tc<FMT_BF16>(*B, lam, st);
     dm_count_launches(1);
