@@ -299,9 +299,10 @@ constexpr unsigned WAIT_HINT_NS = 1000000u;
 
 // Launch shapes the autotuner chooses among (every choice computes identical
 // results): M-tiles of 128 patches per work unit of the tensor-core level-0
-// kernel, pooled rows per CTA tile of the level kernel (8 or 16), CTAs per SM
-// of the backtracking expansion kernels, child-window columns in the level
-// kernel's ring (3 or 2: prefetch depth against shared memory per CTA).
+// kernel, pooled rows per CTA tile of the tiled level kernel (16, 8 or 4; 0: the
+// row-streaming kernel at every level), CTAs per SM of the backtracking expansion
+// kernels, child-window columns in the tiled kernel's ring (3 or 2: prefetch depth
+// against shared memory per CTA).
 struct DmTune {
     int m_chunk;
     int level_th;
@@ -310,9 +311,10 @@ struct DmTune {
 };
 // Defaults until tuned: the level-0 work unit holds all M-tiles of the pair
 // (the N-tiles are the units; measured at 1024x436 the most robust choice for
-// BF16) or, for the FP8 form, half of them (its best measured split); tile
-// rows 8 (on 4 warps; 1024x436: 7.79 ms against 8.31 for 16 rows on 8 warps,
-// 8.71 for 4 rows on 2), 8 CTAs per SM for the backtracking, a ring of 2.
+// BF16) or, for the FP8 form, half of them (its best measured split), and fewer
+// where that fills the GPU's last round of units better; for levels on the tiled
+// kernel tiles of 8 rows and a ring of 2 (the fastest shape at 320x240, 640x480 and
+// 1242x375: level_threads); 8 CTAs per SM for the backtracking.
 inline DmTune dm_tune_default(const DmGeom& g, int precision) {
     const int n_mtiles = (g.npatch(0) + 127) / 128;
     return DmTune{precision == DM_FP8_E4M3 ? (n_mtiles + 1) / 2 : n_mtiles, 8, 8, 2};

@@ -89,10 +89,10 @@ __device__ __forceinline__ void store4(float* dst, int stride, float4 v) {
 // memory, and stores to the transposed rows without bank conflicts; the next
 // tile's centroids are in registers before a tile is computed.
 //
-// What bounds it: the packed fmas' operand reads and the shared loads (five
-// wavefronts per warp and component; ten with the eight patches of a thread side by
-// side, where packing alone gave 0.31 -> 0.295 ms).  27904 patches x 1024 centroids:
-// 0.31 -> 0.197 ms, 42 TFLOP/s.
+// What bounds it: the shared loads (five wavefronts per warp and component; the L1
+// pipe runs at 87 % of its rate, issue at 35 %; ten wavefronts with the eight patches of a
+// thread side by side, where packing alone gave 0.31 -> 0.295 ms).  27904 patches x 1024
+// centroids: 0.31 -> 0.197 ms, 42 TFLOP/s.
 __global__ void __launch_bounds__(256, 2) k_km_assign(const float* __restrict__ A, int P0, const float* __restrict__ C,
                                                       int D, int chunk, float* __restrict__ part_s,
                                                       int* __restrict__ part_i) {

@@ -10,29 +10,36 @@
 // divided by n; pooling is on the unrectified average and the power is
 // applied to the pooled value (x -> x^lambda is increasing on [0,1]).
 //
-// This pass streams the pooled maps of the level below and does a fixed
-// amount of arithmetic per stored output (~4 averages of 4 values, a 9-way
-// max with argmax, one power).  A CTA owns a tile of 32 x TH pooled outputs
-// (TH = 8 by default on 4 warps; 16 on 8 or 4 on 2, autotuned) of a run of up
-// to 32 lattice patches on one row,
-// spaced so that the right child column of one patch is the left child column
-// of the next: the child windows (72 x (2 TH + 1) floats, which cover both
+// The pass reads the pooled maps of the level below and does a fixed amount of
+// arithmetic per stored output (~4 averages of 4 values, a 9-way max with argmax, one
+// power).  Algorithmic bytes per stored output: 16 B of child values read (each child
+// value is shared by 4 parents), 4 + 1 B written.  Two kernels do it, with the same bits;
+// level_streams below says which takes a level, and with what times on either side:
+//
+// k_level_rows, the row-streaming kernel: a warp walks down the rows of its patches' maps
+// in registers, in strips of 64 columns (or of 32, 16 or 8).  It takes the maps that fill
+// its strips, those of at most 16 columns, and small images: every level of 1024x436 and
+// of 512x224.  Described where it stands.
+//
+// k_level_sweep, the tiled kernel: the maps that leave strips part-empty (640x480 levels 1
+// to 4, 1242x375 levels 2 to 5, 320x240 levels 1 to 3; of small images where the maps are
+// wider than 64 columns or another tile than the default was set), and fault injection.  A CTA owns a tile of 32 x TH pooled outputs (TH = 8 by
+// default on 4 warps; 16 on 8 or 4 on 2 as tuned shapes) of a run of up to 32 lattice
+// patches on one row, spaced so that the right child column of one patch is the left
+// child column of the next: the child windows (72 x (2 TH + 1) floats, which cover both
 // shifts +-1 of a shared column) are staged in shared memory by 3-D TMA tensor
-// loads into a ring of NR = 2 (or 3, autotuned) columns; as soon as a patch's
+// loads into a ring of NR = 2 (or 3, as a tuned shape) columns; as soon as a patch's
 // averages are formed its left column is released and one thread starts the
 // loads of the column NR ahead, which overlap the pooling and rectification.
 // Each child window reaches shared memory about twice per (up to) four parents
 // instead of four times; the CTAs of one tile row and one row of patches run
 // together, so the second staging (by the next row of patches) and the window
-// edges shared by neighbouring tiles come from L2, and the maps are read from
-// DRAM about 1.1 times.
+// edges shared by neighbouring tiles come from L2.
 // Every thread forms the same number of averages and of pooled outputs per
 // patch (the CTA meets a barrier after each phase).
 // (Rows of the pooled maps are padded to 16 floats and the window's first
 // column is a multiple of 4, so every load starts 16-byte aligned; the tensor
-// map zero-fills whatever lies outside the domain.)  Algorithmic bytes per
-// stored output: 16 B of child values read (each child value is shared by 4
-// parents), 4 + 1 B written.
+// map zero-fills whatever lies outside the domain.)
 #include <algorithm>
 
 #include "dm_internal.cuh"
@@ -129,13 +136,14 @@ constexpr int AWP = 68;                          // padded row of the averages (
 constexpr int LEVEL_THREADS = 256;
 // threads of a tiled level CTA for TH pooled rows: 8 warps for 16 rows, 4 for 8,
 // 2 for 4 -- every thread forms two 4-column average groups and two pooled
-// outputs per patch, and smaller CTAs wait less at their per-patch barriers
-// (1024x436 levels: 8 rows on 4 warps 7.79 ms, 16 rows on 8 warps 8.30, 8 rows
-// on 8 warps 10.31)
+// outputs per patch, and smaller CTAs wait less at their per-patch barriers.
+// A BF16 pyramid (rows, ring columns; us): 640x480, four of seven levels tiled, 8 2 6279,
+// 8 3 6547, 16 2 6606, 16 3 6884, 4 2 6763, 4 3 7121; 320x240 627, 643, 653, 666, 672, 695;
+// 1242x375 14418, 14569, 14704, 14869, 14694, 14924 (row-streaming at every level: 6792, 659, 14790)
 template <int TH>
 __host__ __device__ constexpr int level_threads() { return TH == 16 ? 256 : (TH == 8 ? 128 : 64); }
 
-// CTA tile of TW x TH pooled outputs (TH = 8 or 16, chosen by the autotuner):
+// CTA tile of TW x TH pooled outputs (TH = 8, 16 or 4):
 // AH rows of averages, child windows of KW x AH floats (KIDF with padding to
 // 128 bytes), KID_BYTES delivered by one TMA window load.
 template <int TH_>
@@ -154,9 +162,9 @@ constexpr long long LEVEL_WAIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
 // Children with o_x = -1 (left, windows lt / lb) read columns ax+2 .. ax+5 (two
 // aligned float4 loads, which unlike 8-byte loads at a 16-byte stride are free
 // of bank conflicts), children with o_x = +1 (right, rt / rb) columns
-// ax+4 .. ax+7.  Then times w = 1/n (n is 1, 2 or 4: valid_all).  Two columns per packed FP32x2 operation: Knuth's TwoSum (6
-// additions, every step correctly rounded per lane) costs 3 instructions per
-// column and step.
+// ax+4 .. ax+7.  Then times w = 1/n (n is 1, 2 or 4: valid_all).  Two columns per packed
+// FP32x2 operation: Knuth's TwoSum (6 additions, every step correctly rounded per lane)
+// costs 3 instructions per column and step.
 template <bool COMP>
 __device__ __forceinline__ float4 avg_group(const float* lt, const float* lb, const float* rt, const float* rb, float w) {
     const float4 a0 = *reinterpret_cast<const float4*>(lt), b0 = *reinterpret_cast<const float4*>(lt + 4);
@@ -196,7 +204,8 @@ __device__ __forceinline__ float2 avg_two(const float* lt, const float* lb, cons
 // iy - e, iy + e' likewise; the stride S = 2^(l-1) (1 at level 1) makes the
 // right column of one patch the left column of the next, so the run needs
 // run + 1 columns of two child windows each instead of 4 windows per patch.
-// Runs of 32 (measured at 1024x436 with 8-row tiles, levels stage: 8 8.09 ms,
+// Runs of 32 (measured at 1024x436 with 8-row tiles at every level wider than 16 columns,
+// which the row-streaming kernel has taken over there, levels stage: 8 8.09 ms,
 // 16 7.79, 32 7.66, 48 7.67, 64 7.63; 32 keeps more CTAs for small images;
 // shorter runs on the small top levels gained nothing).
 __host__ __device__ inline int level_run(int) { return 32; }
@@ -254,10 +263,10 @@ __device__ __forceinline__ void level_sweep_body(const DmGeom& g, int l, const C
     // neighbouring tiles of the row share (64-byte memory granules at their x
     // edges) come from DRAM once, and the next row of patches, which stages the
     // same child rows again, follows within a few hundred CTAs, while they are
-    // still in L2 (1024x436, level 1: DRAM reads 1.14x the maps; all tiles of a
-    // row of patches together instead: 2.1x, their child rows exceed the L2
-    // before the next row of patches reads them again; the tile as the slowest
-    // index: 1.83x at 512x224)
+    // still in L2 (level 1 of 1024x436 on this kernel, tiles of 16 rows: DRAM reads
+    // 1.14x the maps; all tiles of a row of patches together instead: 2.1x, their
+    // child rows exceed the L2 before the next row of patches reads them again; the
+    // tile as the slowest index: 1.83x at 512x224)
     const int rr = item % per_row;
     int t = item / per_row;
     const int tx = t % tiles_x;
