@@ -234,7 +234,8 @@ KmLayout km_layout(const DmGeom& g, int D) {
     l.S = o;    o += dm_align((size_t)D * KD * sizeof(unsigned long long));
     l.cnt = o;  o += dm_align((size_t)D * sizeof(unsigned int));
     l.init = o; o += dm_align((size_t)D * sizeof(int));
-    // centroid chunks: enough CTAs for about three waves of two per SM on 152 SMs
+    // centroid chunks: enough CTAs for about three waves of two per SM on 152 SMs (a number, since the
+    // workspace that a caller has sized may not depend on the device)
     const int P0 = g.P0x * g.P0y;
     const int mblocks = (P0 + KM_BM - 1) / KM_BM;
     const int want = (912 + mblocks - 1) / mblocks;
